@@ -62,7 +62,7 @@ typedef enum {
 
 /* Kernel family used by the expert stage. AUTO picks by L and shape. */
 #define BLOCKFFN_VARIANT_AUTO 0
-#define BLOCKFFN_VARIANT_SIMT 1   /* CUDA-core dot products, fp32 intermediate             */
+#define BLOCKFFN_VARIANT_SIMT 1   /* any shape (d % 8, d_e % 8), fp32 intermediate           */
 #define BLOCKFFN_VARIANT_MMA 2    /* asynchronously staged, tensor-core tiles, bf16 intermediate;
                                      blockffn_create returns UNSUPPORTED for a shape or ring
                                      depth these kernels do not take (d % 64, d_e a power of
@@ -255,7 +255,7 @@ BLOCKFFN_API uint64_t blockffn_launch_count(blockffn_handle h);
 
 /* The paper has no counterpart of this entry point; it exists for deployment reasons only.
  * It is blockffn_expert_ffn (Eq. 1 + Eq. 2 over the listed experts, same arguments, same
- * result as the CUDA-core variant) for callers that are not allowed to allocate device
+ * result as BLOCKFFN_VARIANT_SIMT) for callers that are not allowed to allocate device
  * memory and therefore cannot call blockffn_create, whose workspace comes from cudaMalloc:
  * for instance a plug-in that runs inside a host application which has handed all device
  * memory to its own pool (an allocation would fail, or would stall every stream of the
@@ -264,7 +264,8 @@ BLOCKFFN_API uint64_t blockffn_launch_count(blockffn_handle h);
  * (d, E, d_e, rms_eps unused; L_max, variant and flags are ignored) instead of a handle and
  * makes no call that allocates or frees memory.
  *   - Its intermediate lives in a fixed array inside the library image, which every GPU that
- *     loads the library keeps until the process exits: BLOCKFFN_NOALLOC_SCRATCH_BYTES plus a
+ *     loads the library keeps until the process exits: one and a half times
+ *     BLOCKFFN_NOALLOC_SCRATCH_BYTES (an element is stored as three 16-bit parts) plus a
  *     256-byte header. A call whose E * L * d_e * 4 exceeds that size returns
  *     BLOCKFFN_ERR_WORKSPACE and enqueues nothing.
  *   - The first call on a device looks up the array's device address (with that device

@@ -55,7 +55,8 @@ blockffn_status expert_dispatch(blockffn_ctx* c, const blockffn_weights* w, cons
     e = launch_tensor_core(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, nullptr,
                            nullptr, false, st);
   else
-    e = launch_expert_simt(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, st);
+    e = launch_expert_any(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, nullptr,
+                          nullptr, st);
   return e == cudaSuccess ? BLOCKFFN_OK : BLOCKFFN_ERR_CUDA;
 }
 
@@ -111,7 +112,7 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
     delete c;
     return BLOCKFFN_ERR_CUDA;
   }
-  const size_t E = cfg->E, L = cfg->L_max, d_e = cfg->d_e, W = c->words;
+  const size_t E = cfg->E, L = cfg->L_max, W = c->words;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     size_t o = off;
@@ -126,7 +127,7 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
   const size_t o_um = take(sizeof(uint32_t) * W);
   const size_t o_id = take(sizeof(int32_t) * E);
   const size_t o_nu = take(sizeof(int32_t));
-  const size_t o_h32 = take(sizeof(float) * E * L * d_e);
+  const size_t o_h32 = take(expert_any_h_bytes(cfg));
   const size_t o_h16 = take(expert_mma_h_bytes(cfg));
   const size_t lean_bytes = expert_lean_ws_bytes(cfg, c->num_sms);
   const size_t o_lean = take(lean_bytes);
@@ -155,7 +156,7 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
   c->union_mask = reinterpret_cast<uint32_t*>(b + o_um);
   c->union_ids = reinterpret_cast<int32_t*>(b + o_id);
   c->n_union = reinterpret_cast<int32_t*>(b + o_nu);
-  c->h32 = reinterpret_cast<float*>(b + o_h32);
+  c->h32 = b + o_h32;
   c->h16 = b + o_h16;
   c->lean_ring = lean_bytes ? b + o_lean : nullptr;
   c->lean_seq = reinterpret_cast<unsigned long long*>(b + o_seq);
@@ -170,7 +171,8 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
       return BLOCKFFN_ERR_CUDA;
     }
   }
-  if (expert_mma_setup(c) != cudaSuccess || expert_lean_setup(c) != cudaSuccess) {
+  if (expert_any_setup() != cudaSuccess || expert_mma_setup(c) != cudaSuccess ||
+      expert_lean_setup(c) != cudaSuccess) {
     cudaFree(base);
     delete c;
     return BLOCKFFN_ERR_CUDA;
@@ -221,7 +223,7 @@ blockffn_status blockffn_router(blockffn_handle h, const blockffn_weights* w, co
       (reinterpret_cast<uintptr_t>(tok_mask) & 3u))
     return BLOCKFFN_ERR_INVALID_ARG;
   cudaError_t e =
-      launch_router(h, w, x, L, scores, tok_mask, false, nullptr, false, h->a0, 0,
+      launch_router(h, w, x, L, scores, tok_mask, false, h->a0, 0,
                     static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? BLOCKFFN_OK : BLOCKFFN_ERR_CUDA;
 }
@@ -329,7 +331,7 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     }
     if (aside) {
       if (cudaStreamWaitEvent(side, h->ev_call[oldest], 0) != cudaSuccess ||
-          launch_router(h, w, x, L, h->scores, h->tok_mask, false, nullptr, true, logits, 2,
+          launch_router(h, w, x, L, h->scores, h->tok_mask, true, logits, 2,
                         side) != cudaSuccess ||
           cudaEventRecord(h->ev_router[b], side) != cudaSuccess ||
           cudaStreamWaitEvent(st, h->ev_router[b], 0) != cudaSuccess)
@@ -346,7 +348,7 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     // before it ended, and so does every kernel).
     const bool ahead = x_stable && h->last_layer_waited_first;
     h->last_layer_waited_first = true;
-    if (launch_router(h, w, x, L, h->scores, h->tok_mask, false, nullptr, true, logits,
+    if (launch_router(h, w, x, L, h->scores, h->tok_mask, true, logits,
                       ahead ? 1 : 0, st) != cudaSuccess)
       return BLOCKFFN_ERR_CUDA;
     return launch_tensor_core(h, w, x, h->scores, L, nullptr, nullptr, out, x_next, flags, &pub, &lg,
@@ -355,9 +357,15 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
                : BLOCKFFN_ERR_CUDA;
   }
   h->last_layer_waited_first = false;
-  if (launch_router(h, w, x, L, h->scores, h->tok_mask, true, stats, false, h->a0, 0, st) != cudaSuccess)
+  // Any other shape: the router leaves raw logits, which the expert kernels finish as above.
+  if (launch_router(h, w, x, L, h->scores, h->tok_mask, true, h->a0, 0, st) != cudaSuccess)
     return BLOCKFFN_ERR_CUDA;
-  return expert_dispatch(h, w, x, h->scores, L, h->union_ids, h->n_union, out, x_next, flags, st);
+  const RoutingOut pub{h->union_mask, h->union_ids, h->n_union, stats, h->scores, h->tok_mask};
+  const RouterLogits lg{h->a0, router_gain(h, w), h->cfg.rms_eps};
+  return launch_expert_any(h, w, x, h->scores, L, nullptr, nullptr, out, x_next, flags, &pub, &lg,
+                           st) == cudaSuccess
+             ? BLOCKFFN_OK
+             : BLOCKFFN_ERR_CUDA;
 }
 
 blockffn_status blockffn_layer_forward_scores(blockffn_handle h, const blockffn_weights* w,
@@ -383,12 +391,11 @@ blockffn_status blockffn_layer_forward_scores(blockffn_handle h, const blockffn_
                ? BLOCKFFN_OK
                : BLOCKFFN_ERR_CUDA;
   }
-  if (launch_chunk_union(h, scores, L, h->union_mask, h->union_ids, h->n_union, stats, st) !=
-      cudaSuccess)
-    return BLOCKFFN_ERR_CUDA;
-  // The union list is produced inside this call: the expert stage must wait for it.
-  const int flags = call_flags & ~(BLOCKFFN_CALL_INDEPENDENT | BLOCKFFN_CALL_INDEPENDENT_X);
-  return expert_dispatch(h, w, x, scores, L, h->union_ids, h->n_union, out, x_next, flags, st);
+  const RoutingOut pub{h->union_mask, h->union_ids, h->n_union, stats, nullptr, nullptr};
+  return launch_expert_any(h, w, x, scores, L, nullptr, nullptr, out, x_next, call_flags, &pub,
+                           nullptr, st) == cudaSuccess
+             ? BLOCKFFN_OK
+             : BLOCKFFN_ERR_CUDA;
 }
 
 blockffn_status blockffn_read_routing(blockffn_handle h, int32_t L, float* scores,

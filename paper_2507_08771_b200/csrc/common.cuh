@@ -41,7 +41,7 @@ struct blockffn_ctx {
   uint32_t* union_mask; // [words]
   int32_t* union_ids;   // [E]
   int32_t* n_union;     // [1]
-  float* h32;           // [E][L_max][d_e] fp32 intermediate (SIMT variant)
+  void* h32;            // 32-bit intermediate: three bf16 planes of E L_max d_e (any shape)
   void* h16;            // bf16 intermediate (MMA variant), slot-major padded rows
   void* lean_ring;      // rings of bf16 intermediates of the one-kernel form, then its rings of
                         // router logits (NULL: not used)
@@ -75,8 +75,7 @@ inline const float* router_gain(const blockffn_ctx* c, const blockffn_weights* w
 
 // ---- launchers (each returns the cudaError_t of its launch) ----------------
 cudaError_t launch_router(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
-                          float* scores, uint32_t* tok_mask, bool fuse_union,
-                          blockffn_stats* stats, bool raw, float* logits, int mode,
+                          float* scores, uint32_t* tok_mask, bool raw, float* logits, int mode,
                           cudaStream_t st);
 // mode: 0 the kernel waits for the work before it first; 1 (raw only) it computes under that
 // work and waits at its end; 2 (raw only) it is launched without programmatic chaining on a
@@ -86,11 +85,6 @@ cudaError_t launch_chunk_union(blockffn_ctx* c, const float* scores, int L, uint
                                cudaStream_t st);
 cudaError_t launch_reuse_ratio(blockffn_ctx* c, const float* scores, int L, double* reuse,
                                cudaStream_t st);
-cudaError_t launch_expert_simt(blockffn_ctx* c, const blockffn_weights* w, const void* x,
-                               const float* scores, int L, const int32_t* union_ids,
-                               const int32_t* n_union, float* out, void* x_next, int call_flags,
-                               cudaStream_t st);
-
 // Where a kernel that derives Union(x) itself publishes it (each pointer may be NULL).
 struct RoutingOut {
   uint32_t* union_mask;
@@ -106,6 +100,15 @@ struct RouterLogits {
   const float* gain;    // [E]
   float eps;
 };
+
+// Expert stage for any shape, with a 32-bit intermediate (expert_any.cu). union_ids == NULL: the
+// kernels derive the union from scores, or from raw router logits, and publish it through pub.
+size_t expert_any_h_bytes(const blockffn_config* cfg);
+cudaError_t expert_any_setup();
+cudaError_t launch_expert_any(blockffn_ctx* c, const blockffn_weights* w, const void* x,
+                              const float* scores, int L, const int32_t* union_ids,
+                              const int32_t* n_union, float* out, void* x_next, int call_flags,
+                              const RoutingOut* pub, const RouterLogits* logits, cudaStream_t st);
 
 // One-kernel form of the tensor-core expert stage for chunks of at most 8 tokens (same
 // arguments as launch_expert_mma below).

@@ -302,6 +302,48 @@ __device__ int derive_union(const float* scores, const RouterLogits& lg, const i
   return ctl[0];
 }
 
+// What one CTA (all threads) publishes of the routing it derived; MODE as derive_union.
+template <int MODE>
+__device__ __forceinline__ void publish_routing(const RoutingOut& pub, const RouterLogits& lg, int L,
+                                                int E, int nu, const int* ids_sm, const int* ctl,
+                                                uint32_t* status) {
+  const int tid = threadIdx.x, lane = tid & 31, words = (E + 31) >> 5;
+  if constexpr (MODE == 1) {
+    if (tid == 0 && ctl[3]) atomicOr(status, (uint32_t)ctl[3]);
+    return;
+  }
+  if constexpr (MODE == 2) {      // the scores and masks
+    const float* rinv = reinterpret_cast<const float*>(ctl + 104);
+    for (int t = tid >> 5; pub.scores && t < L; t += blockDim.x >> 5) {
+      for (int w = 0; w < words; ++w) {
+        const int e = 32 * w + lane;
+        float sv = 0.0f;
+        if (e < E) {
+          float v = __ldcg(lg.a0 + (size_t)t * E + e);
+          v = v > 0.0f ? v : 0.0f;
+          sv = __ldg(lg.gain + e) * v * rinv[t];
+          pub.scores[(size_t)t * E + e] = sv;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, sv != 0.0f);
+        if (pub.tok_mask && lane == 0) pub.tok_mask[(size_t)t * words + w] = m;
+      }
+    }
+  }
+  for (int e = tid; e < E; e += blockDim.x) {
+    if (pub.union_ids) pub.union_ids[e] = e < nu ? ids_sm[e] : -1;
+    if (pub.union_mask && e < words) pub.union_mask[e] = (uint32_t)ctl[8 + e];
+  }
+  if (tid == 0) {
+    if (pub.n_union) *pub.n_union = nu;
+    if (pub.stats) {
+      atomicAdd(reinterpret_cast<unsigned long long*>(&pub.stats->n_tokens), (unsigned long long)L);
+      atomicAdd(reinterpret_cast<unsigned long long*>(&pub.stats->n_active), (unsigned long long)ctl[2]);
+      atomicAdd(reinterpret_cast<unsigned long long*>(&pub.stats->n_chunks), 1ull);
+      atomicAdd(reinterpret_cast<unsigned long long*>(&pub.stats->n_union), (unsigned long long)nu);
+    }
+  }
+}
+
 // One 64-wide k block of a 16-row operand tile: rows row_a / row_b (byte addresses of the
 // block within the row), this lane's 16 bytes of each 32-wide half. Lanes of odd rows
 // read the halves in the opposite order (bank spread) and swap them back.

@@ -4,7 +4,7 @@
 // token of the chunk (x . W_r[i] + bias[i]) with 128-bit loads and fp32 FMAs; the
 // block that finishes last (a ticket counter, no waiting) applies ReLU and RMSNorm
 // with the per-expert gain, writes the scores and the per-token nonzero masks
-// (warp ballot), and, for the fused layer call, derives the chunk union right away.
+// (warp ballot).
 //
 // union_kernel: one block ORs the per-token nonzero patterns of a score matrix,
 // compacts the union's expert ids in ascending order with a warp prefix count, and
@@ -79,10 +79,8 @@ __global__ void __launch_bounds__(kThreads)
 router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
               const float* __restrict__ gain, const float* __restrict__ bias, float* a0,
               float* scores, uint32_t* tok_mask, int L, int d, int E, float eps,
-              unsigned int* ticket, int fuse_union, uint32_t* union_mask, int32_t* union_ids,
-              int32_t* n_union, blockffn_stats* stats, int raw, int mode) {
+              unsigned int* ticket, int raw, int mode) {
   __shared__ float red[kWarps][8];
-  __shared__ int sm[3 * kMaxWords];
   __shared__ int is_last;
   const int i = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -196,17 +194,12 @@ router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
       if (tok_mask && lane == 0) tok_mask[(size_t)t * words + w] = m;
     }
   }
-  if (fuse_union) {
-    __syncthreads();
-    chunk_union_block(scores, L, E, union_mask, union_ids, n_union, stats, sm);
-  }
 }
 
 }  // namespace
 
 cudaError_t launch_router(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
-                          float* scores, uint32_t* tok_mask, bool fuse_union,
-                          blockffn_stats* stats, bool raw, float* logits, int mode,
+                          float* scores, uint32_t* tok_mask, bool raw, float* logits, int mode,
                           cudaStream_t st) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -220,9 +213,7 @@ cudaError_t launch_router(blockffn_ctx* c, const blockffn_weights* w, const void
   const cudaError_t e = cudaLaunchKernelEx(
       &lc, router_kernel, static_cast<const uint16_t*>(x), static_cast<const uint16_t*>(w->W_r),
       router_gain(c, w), w->bias, logits, scores, tok_mask, L, c->cfg.d, c->cfg.E, c->cfg.rms_eps,
-      c->ticket,
-      fuse_union ? 1 : 0, c->union_mask, c->union_ids, c->n_union, stats, raw ? 1 : 0,
-      raw ? mode : 0);
+      c->ticket, raw ? 1 : 0, raw ? mode : 0);
   if (e == cudaSuccess) c->launches += 1;
   return e;
 }
