@@ -36,8 +36,7 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
   // which keeps its weights in shared memory for all tokens at once.
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
   const bool dep_long = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
-  const bool dep_inside = !x_stable && logits && logits->a0 == nullptr;   // router inside the kernel
-  if ((x_stable || dep_long || dep_inside) &&
+  if ((x_stable || dep_long) &&
       expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr))
     return launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, pub,
                               logits, logits_final, st);
@@ -132,6 +131,8 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
   const size_t lean_bytes = expert_lean_ws_bytes(cfg, c->num_sms);
   const size_t o_lean = take(lean_bytes);
   const size_t o_seq = take(sizeof(unsigned long long) * 256);   // four rings, 64 words each
+  const size_t chain_bytes = expert_chain_ws_bytes(cfg, c->num_sms);
+  const size_t o_chain = take(chain_bytes);
   const size_t o_one = take(sizeof(float) * E);
   const size_t o_tk = take(sizeof(unsigned int) * 8);
   const size_t o_st = take(sizeof(uint32_t));
@@ -160,6 +161,7 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
   c->h16 = b + o_h16;
   c->lean_ring = lean_bytes ? b + o_lean : nullptr;
   c->lean_seq = reinterpret_cast<unsigned long long*>(b + o_seq);
+  c->chain_ws = chain_bytes ? b + o_chain : nullptr;
   c->ones = reinterpret_cast<float*>(b + o_one);
   c->ticket = reinterpret_cast<unsigned int*>(b + o_tk);
   c->status = reinterpret_cast<uint32_t*>(b + o_st);
@@ -171,8 +173,8 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
       return BLOCKFFN_ERR_CUDA;
     }
   }
-  if (expert_any_setup() != cudaSuccess || expert_mma_setup(c) != cudaSuccess ||
-      expert_lean_setup(c) != cudaSuccess) {
+  if (expert_any_setup(cfg->L_max) != cudaSuccess || expert_mma_setup(c) != cudaSuccess ||
+      expert_lean_setup(c) != cudaSuccess || expert_chain_setup(c) != cudaSuccess) {
     cudaFree(base);
     delete c;
     return BLOCKFFN_ERR_CUDA;
@@ -287,16 +289,22 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     // Successive calls cycle through kLogitRing logit buffers: a router that runs under earlier
     // calls never writes what their kernels still read.
     const bool x_stable_call = (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
-    if (expert_lean_supported(h, L, true, x_stable_call, true)) {
-      // The shape takes the one-kernel form: the router runs inside that kernel (its CTAs share
-      // the experts' logits out between them and exchange them through L2), so the call is one
-      // launch. With x stable it overlaps its neighbours like a scores-in call; otherwise it
-      // owns the device and waits for the work before it ahead of its first read.
-      const RoutingOut pub_in{h->union_mask, h->union_ids, h->n_union, stats, h->scores, h->tok_mask};
+    const RoutingOut pub_in{h->union_mask, h->union_ids, h->n_union, stats, h->scores, h->tok_mask};
+    if (!x_stable_call && expert_chain_supported(h, L)) {
+      // x from the call before: one kernel made for that chain, router included
+      h->last_layer_waited_first = false;
+      return launch_expert_chain(h, w, x, L, out, x_next, call_flags, &pub_in, st) == cudaSuccess
+                 ? BLOCKFFN_OK
+                 : BLOCKFFN_ERR_CUDA;
+    }
+    if (x_stable_call && expert_lean_supported(h, L, true, true, true)) {
+      // x stable: the router runs inside the one-kernel form (its CTAs share the experts' logits
+      // out between them and exchange them through L2), so the call is one launch that overlaps
+      // its neighbours like a scores-in call.
       const RouterLogits lg_in{nullptr, router_gain(h, w), h->cfg.rms_eps};
       h->last_layer_waited_first = false;
       return launch_tensor_core(h, w, x, h->scores, L, nullptr, nullptr, out, x_next, flags, &pub_in,
-                                &lg_in, x_stable_call, st) == cudaSuccess
+                                &lg_in, true, st) == cudaSuccess
                  ? BLOCKFFN_OK
                  : BLOCKFFN_ERR_CUDA;
     }

@@ -48,6 +48,7 @@ struct blockffn_ctx {
   unsigned long long* lean_seq;   // per ring (four of them, 64 words apart): [0] call tickets,
                                   // [1 .. 16] arrival counters of the ring slots, [17 .. 32] those
                                   // of the logit hand-over when the router runs inside the kernel
+  void* chain_ws;       // ticket, logit words and h buffers of the dependent-chain kernel, or NULL
   float* ones;          // [E] of 1.0f: the gain of the router without RMSNorm
   unsigned int* ticket; // last-block-done counters [8]
   uint32_t* status;     // sticky device status word
@@ -104,7 +105,7 @@ struct RouterLogits {
 // Expert stage for any shape, with a 32-bit intermediate (expert_any.cu). union_ids == NULL: the
 // kernels derive the union from scores, or from raw router logits, and publish it through pub.
 size_t expert_any_h_bytes(const blockffn_config* cfg);
-cudaError_t expert_any_setup();
+cudaError_t expert_any_setup(int L_max);
 cudaError_t launch_expert_any(blockffn_ctx* c, const blockffn_weights* w, const void* x,
                               const float* scores, int L, const int32_t* union_ids,
                               const int32_t* n_union, float* out, void* x_next, int call_flags,
@@ -121,6 +122,14 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
                                const int32_t* n_union, float* out, void* x_next, int call_flags,
                                const RoutingOut* pub, const RouterLogits* logits, bool logits_final,
                                cudaStream_t st);
+
+// A whole layer call, router inside, in a dependent chain as one kernel (expert_chain.cu).
+bool expert_chain_supported(const blockffn_ctx* c, int L);
+size_t expert_chain_ws_bytes(const blockffn_config* cfg, int sms);
+cudaError_t expert_chain_setup(blockffn_ctx* c);
+cudaError_t launch_expert_chain(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
+                                float* out, void* x_next, int call_flags, const RoutingOut* pub,
+                                cudaStream_t st);
 
 // Tensor-core / bulk-copy variant of the expert stage. union_ids == NULL: the kernels derive
 // the union from the nonzero pattern of scores and publish it through pub; with logits != NULL

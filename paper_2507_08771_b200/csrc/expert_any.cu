@@ -463,16 +463,16 @@ size_t expert_any_h_bytes(const blockffn_config* cfg) {
   return 3 * sizeof(uint16_t) * (size_t)cfg->E * cfg->L_max * cfg->d_e;
 }
 
-cudaError_t expert_any_setup() {
+cudaError_t expert_any_setup(int L_max) {
   cudaError_t e = any_attr<1, 0>();
   if (e == cudaSuccess) e = any_attr<1, 1>();
   if (e == cudaSuccess) e = any_attr<1, 2>();
-  if (e == cudaSuccess) e = any_attr<2, 0>();
-  if (e == cudaSuccess) e = any_attr<2, 1>();
-  if (e == cudaSuccess) e = any_attr<2, 2>();
-  if (e == cudaSuccess) e = any_attr<4, 0>();
-  if (e == cudaSuccess) e = any_attr<4, 1>();
-  if (e == cudaSuccess) e = any_attr<4, 2>();
+  if (e == cudaSuccess && L_max > 8) e = any_attr<2, 0>();
+  if (e == cudaSuccess && L_max > 8) e = any_attr<2, 1>();
+  if (e == cudaSuccess && L_max > 8) e = any_attr<2, 2>();
+  if (e == cudaSuccess && L_max > 16) e = any_attr<4, 0>();
+  if (e == cudaSuccess && L_max > 16) e = any_attr<4, 1>();
+  if (e == cudaSuccess && L_max > 16) e = any_attr<4, 2>();
   return e;
 }
 
@@ -592,7 +592,7 @@ extern "C" blockffn_status blockffn_expert_ffn_noalloc(
       if (cudaGetSymbolAddress(reinterpret_cast<void**>(&ptr), g_noalloc_scratch) != cudaSuccess ||
           !ptr ||
           cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-          expert_any_setup() != cudaSuccess) {
+          expert_any_setup(32) != cudaSuccess) {
         cudaGetLastError();
         return BLOCKFFN_ERR_CUDA;
       }

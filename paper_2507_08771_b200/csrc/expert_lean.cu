@@ -234,9 +234,6 @@ __global__ void __launch_bounds__(kThreads, 3) expert_lean_kernel(const LeanPara
   if constexpr (MODE == 3) {
     if (tid == 0) on_ticket();
     __syncthreads();
-    // In a dependent chain x (and, without any promise, everything else) is what the call
-    // before leaves: nothing has been read so far, and nothing is before that call is done.
-    if (p.dep) pdl_wait();
     const int rslot = ctl[6];
     float* a0 = p.logit_ring + (size_t)rslot * p.logit_slot;
     lg3.a0 = a0;
@@ -923,21 +920,22 @@ size_t expert_lean_ws_bytes(const blockffn_config* cfg, int sms) {
   return kRings * kHRing * slot;
 }
 
-cudaError_t expert_lean_setup(blockffn_ctx* c) {
-  (void)c;
-  cudaError_t e = lean_attrs_kb<1, 1>();
-  if (e == cudaSuccess) e = lean_attrs_kb<2, 1>();
-  if (e == cudaSuccess) e = lean_attrs_kb<3, 1>();
-  if (e == cudaSuccess) e = lean_attrs_kb<4, 1>();
-  if (e == cudaSuccess) e = lean_attrs_kb<1, 2>();
-  if (e == cudaSuccess) e = lean_attrs_kb<2, 2>();
-  if (e == cudaSuccess) e = lean_attrs_kb<3, 2>();
-  if (e == cudaSuccess) e = lean_attrs_kb<4, 2>();
-  if (e == cudaSuccess) e = lean_attrs_kb<1, 3>();
-  if (e == cudaSuccess) e = lean_attrs_kb<2, 3>();
-  if (e == cudaSuccess) e = lean_attrs_kb<3, 3>();
-  if (e == cudaSuccess) e = lean_attrs_kb<4, 3>();
+// (only the kernels of this handle's width: the first touch of a kernel loads it)
+template <int KB>
+cudaError_t lean_setup_kb() {
+  cudaError_t e = lean_attrs_kb<KB, 1>();
+  if (e == cudaSuccess) e = lean_attrs_kb<KB, 2>();
+  if (e == cudaSuccess) e = lean_attrs_kb<KB, 3>();
   return e;
+}
+cudaError_t expert_lean_setup(blockffn_ctx* c) {
+  if (c->lean_ring == nullptr) return cudaSuccess;
+  switch ((c->cfg.d / 64 + kWarps - 1) / kWarps) {
+    case 1: return lean_setup_kb<1>();
+    case 2: return lean_setup_kb<2>();
+    case 3: return lean_setup_kb<3>();
+    default: return lean_setup_kb<4>();
+  }
 }
 
 cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const void* x,
@@ -948,12 +946,9 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
   // For calls whose x is stable (for a router-on call: whose router has finished), and for
   // chunks of more than 8 tokens in a dependent chain (weights and scores stable, x from the
   // call before): those wait for their predecessor before they read x.
-  // A router-on call of up to 8 tokens whose router runs inside the kernel (logits->a0 == NULL)
-  // may be dependent as well, with or without promises: it waits before it reads anything.
   const bool inside = logits && logits->a0 == nullptr;
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
-  const bool dep = !x_stable &&
-                   (inside || (!logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8));
+  const bool dep = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
   if (!x_stable && !dep) return cudaErrorNotSupported;
   // Nothing consumed from its predecessors: the call shares the device with them (a router-on
   // call is ordered behind its own router by an event, and the routers run far enough ahead on

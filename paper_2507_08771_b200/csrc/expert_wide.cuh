@@ -66,7 +66,6 @@ expert_wide_kernel(const LeanParams p) {
   if constexpr (MODE == 3) {
     if (tid == 0) on_ticket();
     __syncthreads();
-    if (p.dep) pdl_wait();
     const int rslot = ctl[6];
     float* a0 = p.logit_ring + (size_t)rslot * p.logit_slot;
     lg3.a0 = a0;

@@ -104,6 +104,84 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
 }
 __device__ __forceinline__ float swish_fast(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
 
+// Up to 128 experts: ids, count and summary (ctl, as below) of the union from the token masks tm
+// (written before a barrier). Every warp folds the masks itself (lane t holds token t's mask of a
+// word; one warp-wide OR per word), so offsets and the union size need no second exchange through
+// shared memory.
+__device__ __forceinline__ int fold_masks(const uint32_t* tm, int L, int words, int* ids_sm, int* ctl) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t* um = reinterpret_cast<uint32_t*>(ctl + 8);
+  uint32_t un[4];
+  int nact = 0;
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    const uint32_t m = (w < words && lane < L) ? tm[w * 32 + lane] : 0u;
+    un[w] = __reduce_or_sync(0xffffffffu, m);
+    nact += __popc(m);
+  }
+  int off = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    if (w < warp) off += __popc(un[w]);
+    total += __popc(un[w]);
+  }
+  if (warp < words) {
+    uint32_t mine = un[0];
+#pragma unroll
+    for (int w = 1; w < 4; ++w) mine = warp == w ? un[w] : mine;
+    if ((mine >> lane) & 1u) ids_sm[off + __popc(mine & ((1u << lane) - 1u))] = 32 * warp + lane;
+  }
+  if (warp == 4) {    // a warp without a word of its own leaves the summary
+    nact = __reduce_add_sync(0xffffffffu, nact);
+    if (lane < 4) um[lane] = lane == 0 ? un[0] : lane == 1 ? un[1] : lane == 2 ? un[2] : un[3];
+    if (lane == 0) {
+      ctl[0] = total;
+      ctl[2] = nact;
+    }
+  }
+  __syncthreads();
+  return total;
+}
+
+// Likewise for any number of experts.
+__device__ __forceinline__ int union_of_masks(const uint32_t* tm, int L, int words, int* ids_sm, int* ctl) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  int* cnt = ctl + 40;
+  int* act = ctl + 72;
+  uint32_t* um = reinterpret_cast<uint32_t*>(ctl + 8);
+  if (words <= 4) return fold_masks(tm, L, words, ids_sm, ctl);
+  if (threadIdx.x < words) {
+    uint32_t un = 0;
+    int nact = 0;
+    for (int t = 0; t < L; ++t) {
+      const uint32_t m = tm[threadIdx.x * 32 + t];
+      un |= m;
+      nact += __popc(m);
+    }
+    cnt[threadIdx.x] = __popc(un);
+    act[threadIdx.x] = nact;
+    um[threadIdx.x] = un;
+  }
+  __syncthreads();
+  for (int w = warp; w < words; w += nwarps) {
+    int off = 0;
+    for (int v = 0; v < w; ++v) off += cnt[v];
+    const uint32_t un = um[w];
+    if ((un >> lane) & 1u) ids_sm[off + __popc(un & ((1u << lane) - 1u))] = 32 * w + lane;
+  }
+  if (threadIdx.x == 0) {
+    int total = 0, total_act = 0;
+    for (int w = 0; w < words; ++w) {
+      total += cnt[w];
+      total_act += act[w];
+    }
+    ctl[0] = total;
+    ctl[2] = total_act;
+  }
+  __syncthreads();
+  return ctl[0];
+}
+
 // ---- Union(x) inside the CTA -----------------------------------------------------
 // Fills ids_sm[0 .. nu) with the ascending valid expert ids and returns nu. All global
 // loads of one call are independent of each other, so the routine costs one memory latency.
@@ -125,9 +203,6 @@ __device__ int derive_union(const float* scores, const RouterLogits& lg, const i
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
   const int words = (E + 31) >> 5;
-  int* cnt = ctl + 40;
-  int* act = ctl + 72;
-  uint32_t* um = reinterpret_cast<uint32_t*>(ctl + 8);
   float* rinv = reinterpret_cast<float*>(ctl + 104);
   if constexpr (MODE == 2) {
     // Raw router logits: finish Eq. 3 here (ReLU, RMSNorm over all E entries, gain), with the
@@ -203,69 +278,7 @@ __device__ int derive_union(const float* scores, const RouterLogits& lg, const i
   }
   if constexpr (MODE != 1) {
     __syncthreads();
-    if (words <= 4) {
-      // Up to 128 experts every warp folds the token masks itself (lane t holds token t's
-      // mask of a word; one warp-wide OR per word), so offsets and the union size need no
-      // second exchange through shared memory.
-      uint32_t un[4];
-      int nact = 0;
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const uint32_t m = (w < words && lane < L) ? tm[w * 32 + lane] : 0u;
-        un[w] = __reduce_or_sync(0xffffffffu, m);
-        nact += __popc(m);
-      }
-      int off = 0, total = 0;
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        if (w < warp) off += __popc(un[w]);
-        total += __popc(un[w]);
-      }
-      if (warp < words) {
-        uint32_t mine = un[0];
-#pragma unroll
-        for (int w = 1; w < 4; ++w) mine = warp == w ? un[w] : mine;
-        if ((mine >> lane) & 1u) ids_sm[off + __popc(mine & ((1u << lane) - 1u))] = 32 * warp + lane;
-      }
-      if (warp == 4) {    // a warp without a word of its own leaves the summary
-        nact = __reduce_add_sync(0xffffffffu, nact);
-        if (lane < 4) um[lane] = lane == 0 ? un[0] : lane == 1 ? un[1] : lane == 2 ? un[2] : un[3];
-        if (lane == 0) {
-          ctl[0] = total;
-          ctl[2] = nact;
-        }
-      }
-      __syncthreads();
-      return total;
-    }
-    if (threadIdx.x < words) {
-      uint32_t un = 0;
-      int nact = 0;
-      for (int t = 0; t < L; ++t) {
-        const uint32_t m = tm[threadIdx.x * 32 + t];
-        un |= m;
-        nact += __popc(m);
-      }
-      cnt[threadIdx.x] = __popc(un);
-      act[threadIdx.x] = nact;
-      um[threadIdx.x] = un;
-    }
-    __syncthreads();
-    for (int w = warp; w < words; w += nwarps) {
-      int off = 0;
-      for (int v = 0; v < w; ++v) off += cnt[v];
-      const uint32_t un = um[w];
-      if ((un >> lane) & 1u) ids_sm[off + __popc(un & ((1u << lane) - 1u))] = 32 * w + lane;
-    }
-    if (threadIdx.x == 0) {
-      int total = 0, total_act = 0;
-      for (int w = 0; w < words; ++w) {
-        total += cnt[w];
-        total_act += act[w];
-      }
-      ctl[0] = total;
-      ctl[2] = total_act;
-    }
+    return union_of_masks(tm, L, words, ids_sm, ctl);
   } else {
     int n = __ldcg(n_in);
     {
