@@ -18,6 +18,7 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libblockffn.so")
 _lib = None
+_fast = None     # the same entry points without ctypes (csrc/fastcall.cpp), see _load_fast
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_DEVICE = range(6)
 DEV_BAD_UNION_ID, DEV_BAD_UNION_COUNT, DEV_WAIT_EXPIRED = 1, 2, 4
@@ -104,6 +105,18 @@ def load():
     return lib
 
 
+def _load_fast():
+    """The native argument unpacking for the calls a program makes over and over. Its functions
+    return NotImplemented for arguments that are not plain (a stream object, an int for a pointer, a
+    tensor that is not contiguous, ...): those calls go through ctypes."""
+    global _fast
+    load()
+    from . import _fastcall
+    _fastcall.set_types(ctypes.c_void_p, Weights, Config)
+    _fast = _fastcall
+    return _fast
+
+
 def status_string(code: int) -> str:
     return load().blockffn_status_string(int(code)).decode()
 
@@ -146,57 +159,82 @@ def blockffn_destroy(h):
 
 
 def blockffn_router(h, w: Weights, x, L, scores, tok_mask=None, stream=None):
-    _check(load().blockffn_router(h, ctypes.byref(w), _ptr(x), L, _ptr(scores), _ptr(tok_mask),
-                                  _stream(stream)), "blockffn_router")
+    code = (_fast or _load_fast()).router(h, w, x, L, scores, tok_mask, stream)
+    if code is NotImplemented:
+        code = load().blockffn_router(h, ctypes.byref(w), _ptr(x), L, _ptr(scores), _ptr(tok_mask),
+                                      _stream(stream))
+    _check(code, "blockffn_router")
 
 
 def blockffn_chunk_union(h, scores, L, union_mask, union_ids, n_union, stats=None, stream=None):
-    _check(load().blockffn_chunk_union(h, _ptr(scores), L, _ptr(union_mask), _ptr(union_ids),
-                                       _ptr(n_union), _ptr(stats), _stream(stream)),
-           "blockffn_chunk_union")
+    code = (_fast or _load_fast()).chunk_union(h, scores, L, union_mask, union_ids, n_union, stats,
+                                               stream)
+    if code is NotImplemented:
+        code = load().blockffn_chunk_union(h, _ptr(scores), L, _ptr(union_mask), _ptr(union_ids),
+                                           _ptr(n_union), _ptr(stats), _stream(stream))
+    _check(code, "blockffn_chunk_union")
 
 
 def blockffn_expert_ffn(h, w: Weights, x, scores, L, union_ids, n_union, out, x_next=None,
                         call_flags=0, stream=None):
-    _check(load().blockffn_expert_ffn(h, ctypes.byref(w), _ptr(x), _ptr(scores), L,
-                                      _ptr(union_ids), _ptr(n_union), _ptr(out), _ptr(x_next),
-                                      call_flags, _stream(stream)), "blockffn_expert_ffn")
+    code = (_fast or _load_fast()).expert_ffn(h, w, x, scores, L, union_ids, n_union, out, x_next,
+                                              call_flags, stream)
+    if code is NotImplemented:
+        code = load().blockffn_expert_ffn(h, ctypes.byref(w), _ptr(x), _ptr(scores), L,
+                                          _ptr(union_ids), _ptr(n_union), _ptr(out), _ptr(x_next),
+                                          call_flags, _stream(stream))
+    _check(code, "blockffn_expert_ffn")
 
 
 def blockffn_expert_ffn_noalloc(cfg: Config, w: Weights, x, scores, L, union_ids, n_union, out,
                                 x_next=None, call_flags=0, stream=None):
     """Expert stage for callers that may not allocate device memory: no handle, the
     intermediate lives in a fixed array inside the library (see the header for its limits)."""
-    _check(load().blockffn_expert_ffn_noalloc(ctypes.byref(cfg), ctypes.byref(w), _ptr(x),
-                                              _ptr(scores), L, _ptr(union_ids), _ptr(n_union),
-                                              _ptr(out), _ptr(x_next), call_flags,
-                                              _stream(stream)), "blockffn_expert_ffn_noalloc")
+    code = (_fast or _load_fast()).expert_ffn_noalloc(cfg, w, x, scores, L, union_ids, n_union, out,
+                                                      x_next, call_flags, stream)
+    if code is NotImplemented:
+        code = load().blockffn_expert_ffn_noalloc(ctypes.byref(cfg), ctypes.byref(w), _ptr(x),
+                                                  _ptr(scores), L, _ptr(union_ids), _ptr(n_union),
+                                                  _ptr(out), _ptr(x_next), call_flags,
+                                                  _stream(stream))
+    _check(code, "blockffn_expert_ffn_noalloc")
 
 
 def blockffn_layer_forward(h, w: Weights, x, L, out, x_next=None, stats=None, call_flags=0,
                            stream=None):
-    _check(load().blockffn_layer_forward(h, ctypes.byref(w), _ptr(x), L, _ptr(out), _ptr(x_next),
-                                         _ptr(stats), call_flags, _stream(stream)),
-           "blockffn_layer_forward")
+    code = (_fast or _load_fast()).layer_forward(h, w, x, L, out, x_next, stats, call_flags, stream)
+    if code is NotImplemented:
+        code = load().blockffn_layer_forward(h, ctypes.byref(w), _ptr(x), L, _ptr(out), _ptr(x_next),
+                                             _ptr(stats), call_flags, _stream(stream))
+    _check(code, "blockffn_layer_forward")
 
 
 def blockffn_layer_forward_scores(h, w: Weights, x, scores, L, out, x_next=None, stats=None,
                                   call_flags=0, stream=None):
-    _check(load().blockffn_layer_forward_scores(h, ctypes.byref(w), _ptr(x), _ptr(scores), L,
-                                                _ptr(out), _ptr(x_next), _ptr(stats), call_flags,
-                                                _stream(stream)), "blockffn_layer_forward_scores")
+    code = (_fast or _load_fast()).layer_forward_scores(h, w, x, scores, L, out, x_next, stats,
+                                                        call_flags, stream)
+    if code is NotImplemented:
+        code = load().blockffn_layer_forward_scores(h, ctypes.byref(w), _ptr(x), _ptr(scores), L,
+                                                    _ptr(out), _ptr(x_next), _ptr(stats), call_flags,
+                                                    _stream(stream))
+    _check(code, "blockffn_layer_forward_scores")
 
 
 def blockffn_read_routing(h, L, scores=None, tok_mask=None, union_mask=None, union_ids=None,
                           n_union=None, stream=None):
-    _check(load().blockffn_read_routing(h, L, _ptr(scores), _ptr(tok_mask), _ptr(union_mask),
-                                        _ptr(union_ids), _ptr(n_union), _stream(stream)),
-           "blockffn_read_routing")
+    code = (_fast or _load_fast()).read_routing(h, L, scores, tok_mask, union_mask, union_ids, n_union,
+                                                stream)
+    if code is NotImplemented:
+        code = load().blockffn_read_routing(h, L, _ptr(scores), _ptr(tok_mask), _ptr(union_mask),
+                                            _ptr(union_ids), _ptr(n_union), _stream(stream))
+    _check(code, "blockffn_read_routing")
 
 
 def blockffn_reuse_ratio(h, scores, L, reuse, stream=None):
-    _check(load().blockffn_reuse_ratio(h, _ptr(scores), L, _ptr(reuse), _stream(stream)),
-           "blockffn_reuse_ratio")
+    code = (_fast or _load_fast()).reuse_ratio(h, scores, L, reuse, stream)
+    if code is NotImplemented:
+        code = load().blockffn_reuse_ratio(h, _ptr(scores), L, _ptr(reuse), _stream(stream))
+    _check(code, "blockffn_reuse_ratio")
 
 
 def blockffn_last_status(h, clear=False, stream=None) -> int:
@@ -284,6 +322,12 @@ class Layer:
     def _routing(self, L, with_scores):
         """What the last layer call derived, copied out of the handle's workspace."""
         dev = self.device
+        if dev.type == "cuda":
+            bufs = _fast.routing_buffers(L, self.E, self.words, int(with_scores),
+                                         -1 if dev.index is None else dev.index)
+            if bufs is not NotImplemented:
+                blockffn_read_routing(self.h, L, *bufs)
+                return bufs
         scores = torch.empty(L, self.E, dtype=torch.float32, device=dev) if with_scores else None
         tok = torch.empty(L, self.words, dtype=torch.int32, device=dev) if with_scores else None
         um = torch.empty(self.words, dtype=torch.int32, device=dev)

@@ -1,0 +1,50 @@
+"""The native argument unpacking: what is not plain goes through ctypes, which accepts or refuses."""
+import ctypes
+
+import pytest
+import torch
+
+from paper_2507_08771_b200 import binding as B
+
+
+def test_what_is_not_plain_is_left_to_ctypes():
+    fast = B._load_fast()
+    h, w, t = ctypes.c_void_p(0), B.make_weights(), torch.zeros(8)
+    plain = [h, w, None, 1, None, None, None, 0, None]
+    for i, odd in [(0, 0), (0, None), (1, None), (1, h), (2, t), (2, 64), (2, t[::2]), (3, 1.0), (3, True),
+                   (3, 1 << 40), (4, torch.nn.Parameter(t)), (7, None), (8, 0)]:
+        args = list(plain)
+        args[i] = odd
+        assert fast.layer_forward(*args) is NotImplemented, (i, odd)
+    with pytest.raises(TypeError):
+        fast.layer_forward(h)
+    with pytest.raises(AssertionError):       # as before: a CPU tensor is refused
+        B.blockffn_router(h, w, t, 1, t)
+    with pytest.raises(B.BlockFFNError) as e:  # a handle that is NULL
+        B.blockffn_router(h, w, None, 1, None)
+    assert e.value.code == B.ERR_INVALID_ARG
+
+
+@pytest.mark.gpu
+def test_both_ways_give_the_same():
+    d, E, L = 256, 40, 5
+    layer = B.Layer(d, E, 64, L_max=L)
+    x = torch.randn(L, d, device="cuda").bfloat16()
+    W_r = torch.randn(E, d, device="cuda").bfloat16()
+    gain = torch.ones(E, device="cuda")
+    w = B.make_weights(W_r, gain)
+    want, got = torch.zeros(L, E, device="cuda"), torch.zeros(L, E, device="cuda")
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    B.blockffn_router(layer.h, w, x.data_ptr(), L, want.data_ptr(), stream=side)     # ctypes
+    side.synchronize()
+    with torch.cuda.stream(side):
+        B.blockffn_router(layer.h, w, x, L, got)                                     # native, its stream
+    side.synchronize()
+    assert torch.equal(want, got) and bool((got > 0).any())
+    with pytest.raises(AssertionError):
+        B.blockffn_router(layer.h, w, x.t(), L, got)
+    bufs = layer._routing(L, True)
+    assert [tuple(b.shape) for b in bufs] == [(L, E), (L, 2), (2,), (E,), (1,)]
+    assert [b.dtype for b in bufs] == [torch.float32] + 4 * [torch.int32]
+    assert [b is None for b in layer._routing(L, False)] == [True, True, False, False, False]
