@@ -18,11 +18,6 @@ def test_what_is_not_plain_is_left_to_ctypes():
         assert fast.layer_forward(*args) is NotImplemented, (i, odd)
     with pytest.raises(TypeError):
         fast.layer_forward(h)
-    with pytest.raises(AssertionError):       # as before: a CPU tensor is refused
-        B.blockffn_router(h, w, t, 1, t)
-    with pytest.raises(B.BlockFFNError) as e:  # a handle that is NULL
-        B.blockffn_router(h, w, None, 1, None)
-    assert e.value.code == B.ERR_INVALID_ARG
 
 
 @pytest.mark.gpu
@@ -44,6 +39,11 @@ def test_both_ways_give_the_same():
     assert torch.equal(want, got) and bool((got > 0).any())
     with pytest.raises(AssertionError):
         B.blockffn_router(layer.h, w, x.t(), L, got)
+    with pytest.raises(AssertionError):        # a CPU tensor
+        B.blockffn_router(layer.h, w, x.cpu(), L, got)
+    with pytest.raises(B.BlockFFNError) as e:  # a handle that is NULL
+        B.blockffn_router(ctypes.c_void_p(0), w, x, L, got)
+    assert e.value.code == B.ERR_INVALID_ARG
     bufs = layer._routing(L, True)
     assert [tuple(b.shape) for b in bufs] == [(L, E), (L, 2), (2,), (E,), (1,)]
     assert [b.dtype for b in bufs] == [torch.float32] + 4 * [torch.int32]
