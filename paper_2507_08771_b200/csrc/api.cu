@@ -412,6 +412,12 @@ blockffn_status blockffn_read_routing(blockffn_handle h, int32_t L, float* score
   blockffn_status s = check_call(h, L);
   if (s != BLOCKFFN_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (((reinterpret_cast<uintptr_t>(scores) | reinterpret_cast<uintptr_t>(tok_mask) |
+        reinterpret_cast<uintptr_t>(union_mask) | reinterpret_cast<uintptr_t>(union_ids) |
+        reinterpret_cast<uintptr_t>(n_union)) & 3u) == 0)
+    return launch_copy_routing(h, L, scores, tok_mask, union_mask, union_ids, n_union, st) == cudaSuccess
+               ? BLOCKFFN_OK
+               : BLOCKFFN_ERR_CUDA;
   const size_t E = h->cfg.E, W = h->words;
   cudaError_t e = cudaSuccess;
   auto copy = [&](void* dst, const void* src, size_t n) {

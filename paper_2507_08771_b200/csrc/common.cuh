@@ -84,6 +84,9 @@ cudaError_t launch_router(blockffn_ctx* c, const blockffn_weights* w, const void
 cudaError_t launch_chunk_union(blockffn_ctx* c, const float* scores, int L, uint32_t* union_mask,
                                int32_t* union_ids, int32_t* n_union, blockffn_stats* stats,
                                cudaStream_t st);
+cudaError_t launch_copy_routing(blockffn_ctx* c, int L, float* scores, uint32_t* tok_mask,
+                                uint32_t* union_mask, int32_t* union_ids, int32_t* n_union,
+                                cudaStream_t st);
 cudaError_t launch_reuse_ratio(blockffn_ctx* c, const float* scores, int L, double* reuse,
                                cudaStream_t st);
 // Where a kernel that derives Union(x) itself publishes it (each pointer may be NULL).

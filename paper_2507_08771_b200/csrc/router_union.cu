@@ -1,78 +1,51 @@
-// Router (Eq. 3) and chunk union (Sec. 3.3) kernels.
+// Router (Eq. 3), chunk union (Sec. 3.3), reuse ratio (Sec. 4.1.2) and the copy of routing results.
 //
-// router_kernel: one block per expert computes that expert's logit for every
-// token of the chunk (x . W_r[i] + bias[i]) with 128-bit loads and fp32 FMAs; the
-// block that finishes last (a ticket counter, no waiting) applies ReLU and RMSNorm
-// with the per-expert gain, writes the scores and the per-token nonzero masks
-// (warp ballot).
+// All of them are a few KB of data and a chain of memory latencies: what counts is how many of
+// those follow one another, and that the launch runs under the kernel before (programmatic
+// dependent launch). Each kernel asks for all it reads at once; before, a block went through the
+// tokens one after the other (24 tokens, E = 64, d = 2048, one call
+// after the other from a graph: router 12.05 us, union 3.81, reuse ratio 5.57, copy of the routing results 4.36;
+// now 5.5, 2.0, 2.6 and 1.5).
+//
+// router_kernel: a block computes one expert's logits for 8 tokens (x . W_r[i] + bias[i]) with
+// 128-bit loads and fp32 FMAs; of the blocks with the same tokens the one that finishes last (a
+// ticket counter per 8 tokens, no waiting) applies ReLU and RMSNorm with the per-expert gain,
+// writes the scores and the per-token nonzero masks (warp ballot).
 //
 // union_kernel: one block ORs the per-token nonzero patterns of a score matrix,
 // compacts the union's expert ids in ascending order with a warp prefix count, and
 // advances the TLS / CLS counters (Sec. 2.1).
-#include "common.cuh"
+#include "mma_tiles.cuh"
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
 constexpr int kMaxWords = 32;  // E <= 1024
 
-// All 256 threads of the block take part. sm: >= 3 * kMaxWords ints.
-__device__ void chunk_union_block(const float* scores, int L, int E, uint32_t* union_mask,
-                                  int32_t* union_ids, int32_t* n_union, blockffn_stats* stats,
-                                  int* sm) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int words = (E + 31) >> 5;
-  int* cnt = sm;                                   // popcount of each union word
-  int* act = sm + kMaxWords;                       // active (token, expert) pairs per word
-  uint32_t* um = reinterpret_cast<uint32_t*>(sm + 2 * kMaxWords);
-  for (int w = warp; w < words; w += kWarps) {
-    const int e = 32 * w + lane;
-    uint32_t un = 0;
-    int nact = 0;
-    for (int t = 0; t < L; ++t) {
-      float v = (e < E) ? scores[(size_t)t * E + e] : 0.0f;
-      uint32_t m = __ballot_sync(0xffffffffu, v != 0.0f);
-      un |= m;
-      nact += __popc(m);
-    }
-    if (lane == 0) {
-      cnt[w] = __popc(un);
-      act[w] = nact;
-      um[w] = un;
-      if (union_mask) union_mask[w] = un;
-    }
-  }
-  __syncthreads();
-  int total = 0, total_act = 0;
-  for (int w = 0; w < words; ++w) {
-    total += cnt[w];
-    total_act += act[w];
-  }
-  for (int w = warp; w < words; w += kWarps) {
-    int off = 0;
-    for (int v = 0; v < w; ++v) off += cnt[v];
-    const uint32_t un = um[w];
-    if ((un >> lane) & 1u) union_ids[off + __popc(un & ((1u << lane) - 1u))] = 32 * w + lane;
-  }
-  for (int idx = total + threadIdx.x; idx < E; idx += kThreads) union_ids[idx] = -1;
-  if (threadIdx.x == 0) {
-    *n_union = total;
-    if (stats) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(&stats->n_tokens), (unsigned long long)L);
-      atomicAdd(reinterpret_cast<unsigned long long*>(&stats->n_active),
-                (unsigned long long)total_act);
-      atomicAdd(reinterpret_cast<unsigned long long*>(&stats->n_chunks), 1ull);
-      atomicAdd(reinterpret_cast<unsigned long long*>(&stats->n_union), (unsigned long long)total);
-    }
-  }
+// A launch that may start while the work before it on the stream still runs. These kernels do not
+// let their own dependents go early: a call after them may read what they write (union lists,
+// scores) as a stable input before it waits.
+template <class... P, class... A>
+cudaError_t launch_chained(const blockffn_ctx* c, void (*kernel)(P...), int grid, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(grid);
+  lc.blockDim = dim3(kThreads);
+  lc.stream = st;
+  lc.attrs = attr;
+  lc.numAttrs = (c->cfg.flags & BLOCKFFN_CFG_NO_CHAINING) ? 0 : 1;
+  return cudaLaunchKernelEx(&lc, kernel, args...);
 }
 
 __global__ void __launch_bounds__(kThreads)
-union_kernel(const float* __restrict__ scores, int L, int E, uint32_t* union_mask,
-             int32_t* union_ids, int32_t* n_union, blockffn_stats* stats) {
-  __shared__ int sm[3 * kMaxWords];
-  chunk_union_block(scores, L, E, union_mask, union_ids, n_union, stats, sm);
+union_kernel(const float* scores, int L, int E, RoutingOut pub) {
+  __shared__ __align__(16) int ctl[kCtlBytes / 4];
+  __shared__ int ids[32 * kMaxWords];
+  __shared__ uint32_t tm[32 * kMaxWords];
+  pdl_wait();
+  const int nu = derive_union<0>(scores, RouterLogits{}, nullptr, nullptr, L, E, ids, ctl, tm);
+  publish_routing<0>(pub, RouterLogits{}, L, E, nu, ids, ctl, nullptr);
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -82,7 +55,8 @@ router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
               unsigned int* ticket, int raw, int mode) {
   __shared__ float red[kWarps][8];
   __shared__ int is_last;
-  const int i = blockIdx.x;
+  const int npass = (L + 7) >> 3;                      // passes of 8 tokens
+  const int i = blockIdx.x / npass, pass = blockIdx.x - i * npass, t0 = 8 * pass;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int chunks = d >> 3;
   const uint4* wrow = reinterpret_cast<const uint4*>(W_r + (size_t)i * d);
@@ -98,51 +72,48 @@ router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
   {  // x may still change until the wait is over, but asking L2 for its lines now is harmless
     // (L2 is where writes land too); the blocks share the lines out between them
     const int lines = (L * d * 2 + 127) >> 7;
-    for (int ln = i + (int)gridDim.x * (int)threadIdx.x; ln < lines; ln += gridDim.x * kThreads)
+    for (int ln = blockIdx.x + (int)gridDim.x * (int)threadIdx.x; ln < lines; ln += gridDim.x * kThreads)
       asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(x) + (size_t)ln * 128));
   }
   // mode 1 (raw only): x does not come from the work before and a0 is a buffer that work
   // does not read, so the logits are computed under it; the wait moves to the end.
   if (mode == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 
-  for (int t0 = 0; t0 < L; t0 += 8) {
-    float acc[8];
+  float acc[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) acc[t] = 0.0f;
-    for (int c = threadIdx.x; c < chunks; c += kThreads) {
-      const uint4 wv = c == (int)threadIdx.x ? w_first : __ldg(wrow + c);
-      const uint32_t wp[4] = {wv.x, wv.y, wv.z, wv.w};
-      // all eight token vectors are requested before the first is used: one memory latency
-      uint4 xv[8];
+  for (int t = 0; t < 8; ++t) acc[t] = 0.0f;
+  for (int c = threadIdx.x; c < chunks; c += kThreads) {
+    const uint4 wv = c == (int)threadIdx.x ? w_first : __ldg(wrow + c);
+    const uint32_t wp[4] = {wv.x, wv.y, wv.z, wv.w};
+    // all eight token vectors are requested before the first is used: one memory latency
+    uint4 xv[8];
 #pragma unroll
-      for (int t = 0; t < 8; ++t)
-        xv[t] = t0 + t < L ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(t0 + t) * d) + c)
-                           : make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        const uint32_t xp[4] = {xv[t].x, xv[t].y, xv[t].z, xv[t].w};
-#pragma unroll
-        for (int p = 0; p < 4; ++p) {
-          acc[t] = fmaf(bf16_lo(wp[p]), bf16_lo(xp[p]), acc[t]);
-          acc[t] = fmaf(bf16_hi(wp[p]), bf16_hi(xp[p]), acc[t]);
-        }
-      }
-    }
+    for (int t = 0; t < 8; ++t)
+      xv[t] = t0 + t < L ? __ldcg(reinterpret_cast<const uint4*>(x + (size_t)(t0 + t) * d) + c)
+                         : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      float v = acc[t];
+      const uint32_t xp[4] = {xv[t].x, xv[t].y, xv[t].z, xv[t].w};
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][t] = v;
+      for (int p = 0; p < 4; ++p) {
+        acc[t] = fmaf(bf16_lo(wp[p]), bf16_lo(xp[p]), acc[t]);
+        acc[t] = fmaf(bf16_hi(wp[p]), bf16_hi(xp[p]), acc[t]);
+      }
     }
-    __syncthreads();
-    if (threadIdx.x < 8 && t0 + threadIdx.x < L) {
-      float v = b;
+  }
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) v += red[w][threadIdx.x];
-      a0[(size_t)(t0 + threadIdx.x) * E + i] = v;
-    }
-    __syncthreads();
+  for (int t = 0; t < 8; ++t) {
+    float v = acc[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[warp][t] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < 8 && t0 + threadIdx.x < L) {
+    float v = b;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) v += red[w][threadIdx.x];
+    a0[(size_t)(t0 + threadIdx.x) * E + i] = v;
   }
 
   // raw: the logits are all the caller wants (the tensor-core expert kernels normalise them
@@ -157,41 +128,60 @@ router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
     if (mode == 2) __threadfence();
     return;
   }
-  // last block done: normalise. The ticket is reset for the next call.
+  // the last block of these tokens normalises them, a token per warp. The ticket is reset for the
+  // next call.
   __threadfence();
+  __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned int tk = atomicAdd(ticket, 1u);
-    is_last = (tk == gridDim.x - 1);
-    if (is_last) *ticket = 0u;
+    unsigned int tk = atomicAdd(ticket + pass, 1u);
+    is_last = (tk == (unsigned)E - 1u);
+    if (is_last) ticket[pass] = 0u;
   }
   __syncthreads();
   if (!is_last) return;
   __threadfence();
 
-  const int words = (E + 31) >> 5;
-  for (int t = warp; t < L; t += kWarps) {
-    float ss = 0.0f;
-    for (int e = lane; e < E; e += 32) {
-      float v = __ldcg(a0 + (size_t)t * E + e);
-      v = v > 0.0f ? v : 0.0f;
-      ss = fmaf(v, v, ss);
-    }
+  const int words = (E + 31) >> 5, t = t0 + warp;
+  if (t >= L) return;
+  const bool few = words <= 4;   // logits and gains of a token in registers: one round trip
+  float v4[4], g4[4], ss = 0.0f;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    // eps < 0 marks the router without RMSNorm (Sec. 4.2.3): the ReLU values are the scores
-    // (the host passes a gain of ones)
-    const float r = eps < 0.0f ? 1.0f : 1.0f / sqrtf(ss / (float)E + eps);
+  for (int u = 0; u < 4; ++u) {
+    const int e = 32 * u + lane;
+    v4[u] = few && e < E ? __ldcg(a0 + (size_t)t * E + e) : 0.0f;
+    g4[u] = few && e < E ? gain[e] : 0.0f;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    v4[u] = v4[u] > 0.0f ? v4[u] : 0.0f;
+    ss = fmaf(v4[u], v4[u], ss);
+  }
+  for (int e = lane; !few && e < E; e += 32) {
+    float v = __ldcg(a0 + (size_t)t * E + e);
+    v = v > 0.0f ? v : 0.0f;
+    ss = fmaf(v, v, ss);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  // eps < 0 marks the router without RMSNorm (Sec. 4.2.3): the ReLU values are the scores
+  // (the host passes a gain of ones)
+  const float r = eps < 0.0f ? 1.0f : 1.0f / sqrtf(ss / (float)E + eps);
+  auto put = [&](int w, float s) {
+    const int e = 32 * w + lane;
+    if (e < E) scores[(size_t)t * E + e] = s;
+    const uint32_t m = __ballot_sync(0xffffffffu, s != 0.0f);
+    if (tok_mask && lane == 0) tok_mask[(size_t)t * words + w] = m;
+  };
+  if (few) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (u < words) put(u, g4[u] * v4[u] * r);
+  } else {
     for (int w = 0; w < words; ++w) {
       const int e = 32 * w + lane;
-      float s = 0.0f;
-      if (e < E) {
-        float v = __ldcg(a0 + (size_t)t * E + e);
-        v = v > 0.0f ? v : 0.0f;
-        s = gain[e] * v * r;
-        scores[(size_t)t * E + e] = s;
-      }
-      const uint32_t m = __ballot_sync(0xffffffffu, s != 0.0f);
-      if (tok_mask && lane == 0) tok_mask[(size_t)t * words + w] = m;
+      float v = e < E ? __ldcg(a0 + (size_t)t * E + e) : 0.0f;
+      v = v > 0.0f ? v : 0.0f;
+      put(w, e < E ? gain[e] * v * r : 0.0f);
     }
   }
 }
@@ -205,7 +195,7 @@ cudaError_t launch_router(blockffn_ctx* c, const blockffn_weights* w, const void
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t lc{};
-  lc.gridDim = dim3(c->cfg.E);
+  lc.gridDim = dim3(c->cfg.E * ((L + 7) / 8));
   lc.blockDim = dim3(kThreads);
   lc.stream = st;
   lc.attrs = attr;
@@ -220,46 +210,61 @@ cudaError_t launch_router(blockffn_ctx* c, const blockffn_weights* w, const void
 
 namespace {
 
-// Reuse ratio (Sec. 4.1.2). One block. Warp w takes the pairs w, w + 8, ... of a round of eight; thread 0 then adds the
-// round's ratios to the running sum in token order, so the sum has one summation order.
+constexpr int kPairs = 64;     // token pairs of a round
+
+// Reuse ratio (Sec. 4.1.2). One block. A round takes 65 successive tokens: their nonzero masks (a
+// warp per token, four tokens' loads in flight), the 64 ratios (a thread each), and thread 0 adds
+// them in token order, so the sum has one summation order.
 __global__ void __launch_bounds__(kThreads)
-reuse_ratio_kernel(const float* __restrict__ scores, int L, int E, double* reuse) {
-  __shared__ int n_first[kWarps], n_both[kWarps];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+reuse_ratio_kernel(const float* scores, int L, int E, double* reuse) {
+  __shared__ uint32_t mask[kPairs + 1][kMaxWords];
+  __shared__ double ratio[kPairs];               // negative: the pair does not count
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, words = (E + 31) >> 5;
+  pdl_wait();
   double sum = 0.0, pairs = 0.0;
   if (threadIdx.x == 0) {
     sum = reuse[0];
     pairs = reuse[1];
   }
-  for (int i0 = 0; i0 + 1 < L; i0 += kWarps) {
-    const int i = i0 + warp;
-    int a = 0, b = 0;
-    if (i + 1 < L) {
-      for (int e = lane; e < E; e += 32) {
-        const bool now = scores[(size_t)i * E + e] != 0.0f;
-        const bool next = scores[(size_t)(i + 1) * E + e] != 0.0f;
-        a += now;
-        b += now && next;
+  for (int i0 = 0; i0 + 1 < L; i0 += kPairs) {
+    const int nt = min(kPairs + 1, L - i0);
+    for (int w0 = 0; w0 < words; w0 += 4) {
+      for (int tb = warp; tb < nt; tb += 4 * kWarps) {
+        float v[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int t = tb + j * kWarps, e = 32 * (w0 + u) + lane;
+            v[j][u] = t < nt && e < E ? scores[(size_t)(i0 + t) * E + e] : 0.0f;
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const uint32_t m = __ballot_sync(0xffffffffu, v[j][u] != 0.0f);
+            if (lane == 0 && tb + j * kWarps < nt && w0 + u < words) mask[tb + j * kWarps][w0 + u] = m;
+          }
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    if (lane == 0) {
-      n_first[warp] = a;
-      n_both[warp] = b;
+    __syncthreads();
+    if (threadIdx.x + 1 < nt) {
+      int a = 0, b = 0;
+      for (int w = 0; w < words; ++w) {
+        const uint32_t now = mask[threadIdx.x][w];
+        a += __popc(now);
+        b += __popc(now & mask[threadIdx.x + 1][w]);
+      }
+      ratio[threadIdx.x] = a ? (double)b / (double)a : -1.0;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int w = 0; w < kWarps && i0 + w + 1 < L; ++w) {
-        if (n_first[w] == 0) continue;
-        sum += (double)n_both[w] / (double)n_first[w];
+      for (int k = 0; k + 1 < nt; ++k) {
+        if (ratio[k] < 0.0) continue;
+        sum += ratio[k];
         pairs += 1.0;
       }
     }
-    __syncthreads();
   }
   if (threadIdx.x == 0) {
     reuse[0] = sum;
@@ -267,19 +272,57 @@ reuse_ratio_kernel(const float* __restrict__ scores, int L, int E, double* reuse
   }
 }
 
+// 32-bit words of up to five arrays to the caller's buffers
+struct CopyParams {
+  const uint32_t* src[5];
+  uint32_t* dst[5];
+  uint32_t words[5];
+};
+__global__ void __launch_bounds__(kThreads) copy_routing_kernel(const CopyParams p) {
+  pdl_wait();
+#pragma unroll
+  for (int k = 0; k < 5; ++k)
+    for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < p.words[k]; i += gridDim.x * kThreads)
+      p.dst[k][i] = p.src[k][i];
+}
+
 }  // namespace
 
 cudaError_t launch_reuse_ratio(blockffn_ctx* c, const float* scores, int L, double* reuse,
                                cudaStream_t st) {
-  reuse_ratio_kernel<<<1, kThreads, 0, st>>>(scores, L, c->cfg.E, reuse);
-  c->launches += 1;
-  return cudaGetLastError();
+  const cudaError_t e = launch_chained(c, reuse_ratio_kernel, 1, st, scores, L, (int)c->cfg.E, reuse);
+  if (e == cudaSuccess) c->launches += 1;
+  return e;
 }
 
 cudaError_t launch_chunk_union(blockffn_ctx* c, const float* scores, int L, uint32_t* union_mask,
                                int32_t* union_ids, int32_t* n_union, blockffn_stats* stats,
                                cudaStream_t st) {
-  union_kernel<<<1, kThreads, 0, st>>>(scores, L, c->cfg.E, union_mask, union_ids, n_union, stats);
-  c->launches += 1;
-  return cudaGetLastError();
+  const RoutingOut pub{union_mask, union_ids, n_union, stats, nullptr, nullptr};
+  const cudaError_t e = launch_chained(c, union_kernel, 1, st, scores, L, (int)c->cfg.E, pub);
+  if (e == cudaSuccess) c->launches += 1;
+  return e;
+}
+
+// One kernel instead of a copy per array: a copy of 1 KB takes as long as a launch.
+cudaError_t launch_copy_routing(blockffn_ctx* c, int L, float* scores, uint32_t* tok_mask,
+                                uint32_t* union_mask, int32_t* union_ids, int32_t* n_union,
+                                cudaStream_t st) {
+  const uint32_t E = c->cfg.E, W = c->words;
+  CopyParams p{};
+  const void* src[5] = {c->scores, c->tok_mask, c->union_mask, c->union_ids, c->n_union};
+  void* dst[5] = {scores, tok_mask, union_mask, union_ids, n_union};
+  const uint32_t words[5] = {L * E, L * W, W, E, 1};
+  uint32_t most = 0;
+  for (int k = 0; k < 5; ++k) {
+    p.src[k] = static_cast<const uint32_t*>(src[k]);
+    p.dst[k] = static_cast<uint32_t*>(dst[k]);
+    p.words[k] = dst[k] ? words[k] : 0;
+    if (p.words[k] > most) most = p.words[k];
+  }
+  if (most == 0) return cudaSuccess;
+  const uint32_t blocks = (most + kThreads - 1) / kThreads;
+  const cudaError_t e = launch_chained(c, copy_routing_kernel, (int)(blocks < 32 ? blocks : 32), st, p);
+  if (e == cudaSuccess) c->launches += 1;
+  return e;
 }
