@@ -43,7 +43,7 @@ def parse():
     p.add_argument("--config", type=int, default=1, choices=[1, 2, 3, 4])
     p.add_argument("--L", type=int, default=None, help="chunk length (default: the config's)")
     p.add_argument("--chunks", type=int, default=1024, help="chunks per step")
-    p.add_argument("--variant", type=int, default=0, help="0 auto, 1 CUDA-core, 2 tensor-core")
+    p.add_argument("--variant", type=int, default=0, help="0 auto, 1 any shape (32-bit intermediate), 2 tensor-core tiles")
     p.add_argument("--flags", type=lambda v: int(v, 0), default=0,
                    help="blockffn_config.flags (ring depths, BLOCKFFN_CFG_* bits)")
     p.add_argument("--no-cpu-baseline", action="store_true")
@@ -811,7 +811,7 @@ def extras(args, torch, device, peak):
         assert wl.layer.last_status() == 0
         return ms
 
-    # config 2: L sweep, tensor-core path against CUDA-core path
+    # config 2: L sweep, the tiled tensor-core path against the any-shape path
     rows = []
     for L in I.L_SWEEP:
         row = {"L": L}
