@@ -181,6 +181,13 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
     delete c;
     return BLOCKFFN_ERR_CUDA;
   }
+  // The fills and the copy above ran on the legacy default stream, behind which a caller's
+  // non-blocking stream is not ordered: a handle leaves here with its workspace filled.
+  if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+    cudaFree(base);
+    delete c;
+    return BLOCKFFN_ERR_CUDA;
+  }
   // A caller that names the tensor-core kernels gets them or an error, never a silent switch
   // to the other family (AUTO keeps choosing per call).
   if (cfg->variant == BLOCKFFN_VARIANT_MMA &&

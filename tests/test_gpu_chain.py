@@ -99,3 +99,23 @@ def test_wait_that_runs_out_leaves_the_handle_usable():
         held.forward(dw, x, out=out)
         assert held.last_status(clear=True) == B.DEV_WAIT_EXPIRED
         assert bool((out == 7.0).all())
+
+
+def test_a_new_handle_has_its_workspace_filled():
+    """The first call may come on a stream that is not ordered behind the default one, where
+    blockffn_create fills the workspace (250 MB of "not written yet" here, some 40 us of work)."""
+    h = B.blockffn_create(64, 960, 2048, 32)
+    idle = torch.cuda.default_stream().query()
+    B.blockffn_destroy(h)
+    assert idle
+    d, E, d_e, L = 512, 32, 64, 8
+    dw = make(d, E, d_e, 1, -0.5)
+    x = torch.randn(L, d, device="cuda").bfloat16()
+    _, ref = reference(dw.tensors, x)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        layer, out = B.Layer(d, E, d_e, L_max=L), torch.empty(L, d, device="cuda")
+        B.blockffn_layer_forward(layer.h, dw.struct, x, L, out)
+        torch.cuda.synchronize()
+    assert layer.last_status() == 0
+    assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
