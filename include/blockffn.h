@@ -27,6 +27,14 @@
  *     failures). Problems found on the device (a union id out of range, a count
  *     larger than E) set bits in a sticky status word, skip the offending work and
  *     never fault; read it with blockffn_last_status().
+ *   - Calls whose CTAs exchange data inside one kernel need all CTAs of the call resident at
+ *     once, at most one per SM: blockffn_layer_forward, and scores-in or list calls with one of
+ *     the two promises below (the INDEPENDENT flags). Such calls of two handles on two streams
+ *     are fine while other work lets go of the SMs in time; a call that cannot get its SMs
+ *     within a second gives up (BLOCKFFN_DEV_WAIT_EXPIRED). A program that shares the GPU with
+ *     kernels that hold SMs for that long, or that runs several handles' calls at the same time
+ *     on streams of different priorities, sets BLOCKFFN_CFG_TWO_KERNELS: no kernel then waits
+ *     for another CTA. Scores-in and list calls without a promise never do.
  *   - Limits: 1 <= L <= L_max <= 32 per call; d % 8 == 0; d_e % 8 == 0;
  *     1 <= E <= 1024.
  */
@@ -90,9 +98,11 @@ typedef struct {
  * weights while the kernel enqueued before it on the stream is still finishing
  * (programmatic dependent launch); this bit launches them fully serialised instead. */
 #define BLOCKFFN_CFG_NO_CHAINING 0x10000
-/* A call whose x is stable normally runs as one kernel, several calls in flight per SM; this
- * bit selects the two-kernel form (up projection, down projection), the form every other call
- * takes, for those calls too. Same results within the tolerance; kept for comparison.        */
+/* A call whose x is stable, a router-on layer call and a promised chunk of more than 8 tokens
+ * normally run as one kernel whose CTAs exchange the intermediate (and the router's logits); this
+ * bit selects kernels that follow one another instead (router, up projection, down projection)
+ * for all of them. Same results within the tolerance. For programs that share the GPU, see the
+ * conventions above, and for comparison.                                                    */
 #define BLOCKFFN_CFG_TWO_KERNELS 0x20000000
 /* The one-kernel form runs a call whose x is promised stable (BLOCKFFN_CALL_INDEPENDENT_X) on
  * about a third of the SMs, so that about three times as many such calls are in flight: every CTA reads all

@@ -32,12 +32,13 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
   // router-on call: the router has finished before the expert stage starts). A call of up to 8
   // tokens in a dependent chain (x comes from the call before) runs as the pair, whose two
   // hand-overs are shorter than a grid-wide exchange inside one kernel; a longer chunk in such a
-  // chain takes the one-kernel form on the whole device, which keeps its weights in shared memory
-  // for all tokens at once, with or without promises (no promise, list given, d = 2048, E = 64:
-  // 24 tokens, union 19: 15.4 -> 14.0 us; 32 tokens, union 60: 83 -> 31; 16 tokens, union 19: 11.8
-  // -> 12.0, the worst; 2.8B tree: 39 -> 23; 12 tokens at d = 1536: 9.2 -> 8.4).
+  // chain (weights and scores promised stable) takes the one-kernel form on the whole device,
+  // which keeps its weights in shared memory for all tokens at once. Without a promise it stays
+  // with the pair: the one kernel needs all its CTAs resident at once, and a call that promises
+  // nothing is not to depend on what other streams run (24 tokens, d = 2048, E = 64, union 19, list
+  // given: 15.4 us as the pair, 14.0 as one kernel; 16 tokens 11.2 and 11.6; 32 tokens 18.8 and 14.7).
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
-  const bool dep_long = !x_stable && !logits && L > 8;
+  const bool dep_long = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
   if ((x_stable || dep_long) &&
       expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr))
     return launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, pub,

@@ -1,5 +1,6 @@
 // Expert stage (Eq. 1, Eq. 2 restricted to Union(x), Sec. 3.3) as one kernel per call, for
-// calls whose inputs are all stable (x included), so that several calls are in flight per SM.
+// calls whose inputs are all stable (x included), so that several calls are in flight per SM,
+// and for chunks of more than 8 tokens of which everything but x is promised stable.
 // expert_lean_kernel takes chunks of up to 8 tokens, expert_wide_kernel (expert_wide.cuh) chunks
 // of 9 to 32.
 //
@@ -113,8 +114,7 @@ struct LeanParams {
   uint32_t magic_cpr;          // ceil(2^16 / (d / 8)): tid / (d / 8) = tid * magic_cpr >> 16
   int max_cols, cols_q, cols_rem;
   int accumulate;
-  int dep;                     // x comes from the work before on the stream: wait before reading it
-                               // (1), before reading anything (2)
+  int dep;                     // x comes from the call before on the stream: wait before reading it
   int hold;                    // test aid: wait for an arrival that never comes
   unsigned long long wait_ns;  // bound of the hand-over wait
   uint32_t* status;
@@ -949,7 +949,7 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
   // call before): those wait for their predecessor before they read x.
   const bool inside = logits && logits->a0 == nullptr;
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
-  const int dep = x_stable || logits || L <= 8 ? 0 : (call_flags & BLOCKFFN_CALL_INDEPENDENT) ? 1 : 2;
+  const bool dep = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
   if (!x_stable && !dep) return cudaErrorNotSupported;
   // Nothing consumed from its predecessors: the call shares the device with them (a router-on
   // call is ordered behind its own router by an event, and the routers run far enough ahead on
@@ -1000,7 +1000,7 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
   p.cols_q = pl.cols_q;
   p.cols_rem = pl.cols_rem;
   p.accumulate = (call_flags & BLOCKFFN_CALL_ACCUMULATE) ? 1 : 0;
-  p.dep = dep;
+  p.dep = dep ? 1 : 0;
   p.hold = (c->cfg.flags & BLOCKFFN_CFG_TEST_EXPIRE_WAIT) ? 1 : 0;
   p.wait_ns = 1000000000ull;      // one second
   p.status = c->status;

@@ -44,7 +44,6 @@ expert_wide_kernel(const LeanParams p) {
   const int G = gridDim.x, bx = blockIdx.x;   // the weights are shared out over the CTAs of the call
   const unsigned Gt = gridDim.x;
 
-  if (p.dep == 2) pdl_wait();        // nothing is promised: scores and lists may come from that work
   if (tid < 8) ctl[tid] = 0;
   unsigned long long ticket = 0;
   if (tid == 0) ticket = atomicAdd(p.seq, 1ull);
