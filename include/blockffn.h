@@ -150,7 +150,10 @@ typedef struct {
 #define BLOCKFFN_CALL_INDEPENDENT 2 /* scores, union_ids, n_union and the weights of this call are
                                        stable: nothing enqueued on `stream` since the last call made
                                        without this flag (or since the last host synchronisation)
-                                       writes them. x and out may still come from the work just
+                                       writes them, and neither does that call itself unless it is
+                                       blockffn_chunk_union or blockffn_read_routing (the scores of
+                                       blockffn_router are stable from the second call after it on).
+                                       x and out may still come from the work just
                                        before. The weight fetch then overlaps the previous kernel
                                        (a chunk of more than 8 tokens then runs as one kernel that
                                        waits for that work before it reads x).                      */

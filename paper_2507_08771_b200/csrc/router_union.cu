@@ -22,8 +22,9 @@ namespace {
 constexpr int kMaxWords = 32;  // E <= 1024
 
 // A launch that may start while the work before it on the stream still runs. These kernels do not
-// let their own dependents go early: a call after them may read what they write (union lists,
-// scores) as a stable input before it waits.
+// let their own dependents go early, and fence what they write (union lists, copied scores) before
+// they exit: a call after them may read it as a stable input before it waits, and nothing but the
+// exit of their blocks orders it behind them then.
 template <class... P, class... A>
 cudaError_t launch_chained(const blockffn_ctx* c, void (*kernel)(P...), int grid, cudaStream_t st, A... args) {
   cudaLaunchAttribute attr[1];
@@ -46,6 +47,7 @@ union_kernel(const float* scores, int L, int E, RoutingOut pub) {
   pdl_wait();
   const int nu = derive_union<0>(scores, RouterLogits{}, nullptr, nullptr, L, E, ids, ctl, tm);
   publish_routing<0>(pub, RouterLogits{}, L, E, nu, ids, ctl, nullptr);
+  __threadfence();
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -66,7 +68,10 @@ router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
   // x and everything this kernel writes are touched only after the wait.
   // mode 2 (raw, launched on a stream of its own): dependents are let go only by the exit of
   // the blocks, behind a fence, because they read the logits without waiting (see the end).
-  if (mode != 2) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // raw: the expert kernels that follow wait themselves before they let anything go. A router call
+  // of its own lets its dependents go behind its wait: they may take what was written before it as
+  // stable (the scores of the router call before, say).
+  if (raw && mode != 2) pdl_trigger();
   uint4 w_first = make_uint4(0u, 0u, 0u, 0u);
   if ((int)threadIdx.x < chunks) w_first = __ldg(wrow + threadIdx.x);
   {  // x may still change until the wait is over, but asking L2 for its lines now is harmless
@@ -77,7 +82,8 @@ router_kernel(const uint16_t* __restrict__ x, const uint16_t* __restrict__ W_r,
   }
   // mode 1 (raw only): x does not come from the work before and a0 is a buffer that work
   // does not read, so the logits are computed under it; the wait moves to the end.
-  if (mode == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (mode == 0) pdl_wait();
+  if (!raw) pdl_trigger();
 
   float acc[8];
 #pragma unroll
@@ -284,6 +290,7 @@ __global__ void __launch_bounds__(kThreads) copy_routing_kernel(const CopyParams
   for (int k = 0; k < 5; ++k)
     for (uint32_t i = blockIdx.x * kThreads + threadIdx.x; i < p.words[k]; i += gridDim.x * kThreads)
       p.dst[k][i] = p.src[k][i];
+  __threadfence();
 }
 
 }  // namespace
