@@ -39,7 +39,8 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
   // given: 15.4 us as the pair, 14.0 as one kernel; 16 tokens 11.2 and 11.6; 32 tokens 18.8 and 14.7).
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
   const bool dep_long = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
-  if ((x_stable || dep_long) &&
+  const bool dep_inside = !x_stable && logits && logits->a0 == nullptr;   // router inside the kernel
+  if ((x_stable || dep_long || dep_inside) &&
       expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr))
     return launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, pub,
                               logits, logits_final, st);
@@ -307,14 +308,17 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
                  ? BLOCKFFN_OK
                  : BLOCKFFN_ERR_CUDA;
     }
-    if (x_stable_call && expert_lean_supported(h, L, true, true, true)) {
+    if ((x_stable_call || L > 8) && expert_lean_supported(h, L, true, x_stable_call, true)) {
       // x stable: the router runs inside the one-kernel form (its CTAs share the experts' logits
       // out between them and exchange them through L2), so the call is one launch that overlaps
-      // its neighbours like a scores-in call.
+      // its neighbours like a scores-in call. A dependent call comes here where the score matrix
+      // leaves the chain kernel no room for its pools (17 to 32 tokens of about a thousand experts):
+      // one launch on the whole device. d_e = 64: 117 us per layer at d = 1024, E = 992, 32 tokens
+      // against 243 for the router and the pair; 112 against 171 at d = 2048, E = 800, 24 tokens.
       const RouterLogits lg_in{nullptr, router_gain(h, w), h->cfg.rms_eps};
       h->last_layer_waited_first = false;
       return launch_tensor_core(h, w, x, h->scores, L, nullptr, nullptr, out, x_next, flags, &pub_in,
-                                &lg_in, true, st) == cudaSuccess
+                                &lg_in, x_stable_call, st) == cudaSuccess
                  ? BLOCKFFN_OK
                  : BLOCKFFN_ERR_CUDA;
     }

@@ -945,11 +945,12 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
                                const RoutingOut* pub, const RouterLogits* logits, bool logits_final,
                                cudaStream_t st) {
   // For calls whose x is stable (for a router-on call: whose router has finished), and for
-  // chunks of more than 8 tokens in a dependent chain (weights and scores stable, x from the
-  // call before): those wait for their predecessor before they read x.
+  // chunks of more than 8 tokens in a dependent chain: with scores given (weights and scores
+  // stable, x from the call before) those wait for their predecessor before they read x, with the
+  // router inside before they read anything.
   const bool inside = logits && logits->a0 == nullptr;
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
-  const bool dep = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
+  const bool dep = !x_stable && L > 8 && (inside || (!logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT)));
   if (!x_stable && !dep) return cudaErrorNotSupported;
   // Nothing consumed from its predecessors: the call shares the device with them (a router-on
   // call is ordered behind its own router by an event, and the routers run far enough ahead on

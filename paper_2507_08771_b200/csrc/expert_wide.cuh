@@ -64,6 +64,8 @@ expert_wide_kernel(const LeanParams p) {
   // (a row has at most 256 pieces of 16 bytes: one per thread of a team).
   RouterLogits lg3 = p.lg;
   if constexpr (MODE == 3) {
+    // (a dependent call reads nothing, and lets nothing go, before the work before it is done)
+    if (p.dep) pdl_wait();
     if (tid == 0) on_ticket();
     __syncthreads();
     const int rslot = ctl[6];

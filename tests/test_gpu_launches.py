@@ -3,7 +3,7 @@ import pytest
 import torch
 
 from paper_2507_08771_b200 import binding as B
-from test_gpu_chain import make
+from test_gpu_chain import make, reference
 
 pytestmark = pytest.mark.gpu
 
@@ -33,3 +33,40 @@ def test_calls_without_a_promise_need_no_resident_grid(L):
             torch.cuda.synchronize()
             assert launches(layer, lambda: call(out)) == want
             assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+
+
+@pytest.mark.parametrize("d,E,L,want", [
+    (2048, 544, 32, 1), (1024, 992, 32, 1), (2048, 712, 24, 1), (2048, 952, 17, 1),   # no pools of the chain kernel
+    (512, 1024, 16, 1), (512, 1024, 32, 1),                                           # the chain kernel
+])
+@pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
+def test_dependent_router_on_calls_of_many_experts(d, E, L, want, flags):
+    """One kernel with the router inside, whatever room the score matrix of a chunk takes."""
+    dw, layer = make(d, E, 64, 2, -1.2), B.Layer(d, E, 64, L_max=L)
+    g = torch.Generator(device="cuda").manual_seed(L)
+    h = torch.randn(L, d, device="cuda", generator=g)
+    x = [h.bfloat16(), torch.empty(L, d, dtype=torch.bfloat16, device="cuda")]
+    torch.cuda.synchronize()
+
+    before = h.double()
+    n = layer.launch_count()
+    B.blockffn_layer_forward(layer.h, dw.struct, x[0], L, h, x[1], None, flags | B.CALL_ACCUMULATE)
+    torch.cuda.synchronize()
+    assert layer.launch_count() - n == want and layer.last_status() == 0
+    _, ref = reference(dw.tensors, x[0])
+    assert (h.double() - before - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+    assert torch.equal(x[1], h.bfloat16())
+
+    results = []
+    start = h.clone()
+    for sync in (True, False):   # three layers one after the other, with and without a pause
+        h.copy_(start)
+        x[0].copy_(start)
+        torch.cuda.synchronize()
+        for i in range(3):
+            B.blockffn_layer_forward(layer.h, dw.struct, x[i % 2], L, h, x[(i + 1) % 2], None, flags | B.CALL_ACCUMULATE)
+            if sync:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        results.append(h.clone())
+    assert torch.equal(*results) and layer.last_status() == 0
