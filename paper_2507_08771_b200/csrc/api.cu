@@ -426,9 +426,20 @@ blockffn_status blockffn_read_routing(blockffn_handle h, int32_t L, float* score
   blockffn_status s = check_call(h, L);
   if (s != BLOCKFFN_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (((reinterpret_cast<uintptr_t>(scores) | reinterpret_cast<uintptr_t>(tok_mask) |
-        reinterpret_cast<uintptr_t>(union_mask) | reinterpret_cast<uintptr_t>(union_ids) |
-        reinterpret_cast<uintptr_t>(n_union)) & 3u) == 0)
+  // One kernel where it may write every buffer, i.e. where all of them are 4-byte aligned memory of
+  // the handle's own device; copies otherwise (another GPU's memory, pinned host memory), which need
+  // no mapping into this device. (The look-ups are host work of about 0.2 us a buffer.)
+  auto own = [&](const void* p) {
+    if (!p) return true;
+    if (reinterpret_cast<uintptr_t>(p) & 3u) return false;
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == h->device;
+  };
+  if (own(scores) && own(tok_mask) && own(union_mask) && own(union_ids) && own(n_union))
     return launch_copy_routing(h, L, scores, tok_mask, union_mask, union_ids, n_union, st) == cudaSuccess
                ? BLOCKFFN_OK
                : BLOCKFFN_ERR_CUDA;
