@@ -9,7 +9,10 @@ object has not been built (``python __graft_entry__.py``).
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
+import re
+import warnings
 from dataclasses import dataclass
 
 import numpy as np
@@ -105,15 +108,30 @@ def load():
     return lib
 
 
+class _NoFast:
+    """In the place of the native module: every call goes through ctypes."""
+
+    def __getattr__(self, name):
+        return lambda *args: NotImplemented
+
+
 def _load_fast():
     """The native argument unpacking for the calls a program makes over and over. Its functions
     return NotImplemented for arguments that are not plain (a stream object, an int for a pointer, a
-    tensor that is not contiguous, ...): those calls go through ctypes."""
+    tensor that is not contiguous, ...): those calls go through ctypes. So do all of them, with a
+    warning, where the module is missing or was built for another torch: it only saves host time."""
     global _fast
     load()
-    from . import _fastcall
-    _fastcall.set_types(ctypes.c_void_p, Weights, Config)
-    _fast = _fastcall
+    try:
+        mod = importlib.import_module("._fastcall", __package__)
+        if mod.TORCH_VERSION != re.match(r"\d+\.\d+\.\d+", torch.__version__)[0]:
+            raise ImportError(f"built for torch {mod.TORCH_VERSION}, this is {torch.__version__}")
+        mod.set_types(ctypes.c_void_p, Weights, Config)
+        _fast = mod
+    except ImportError as e:
+        warnings.warn(f"_fastcall is not used ({e}): calls go through ctypes, at 5 to 8 us more host time "
+                      "each; build it with `python __graft_entry__.py`")
+        _fast = _NoFast()
     return _fast
 
 
@@ -323,8 +341,8 @@ class Layer:
         """What the last layer call derived, copied out of the handle's workspace."""
         dev = self.device
         if dev.type == "cuda":
-            bufs = _fast.routing_buffers(L, self.E, self.words, int(with_scores),
-                                         -1 if dev.index is None else dev.index)
+            bufs = (_fast or _load_fast()).routing_buffers(L, self.E, self.words, int(with_scores),
+                                                           -1 if dev.index is None else dev.index)
             if bufs is not NotImplemented:
                 blockffn_read_routing(self.h, L, *bufs)
                 return bufs

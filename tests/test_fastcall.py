@@ -1,5 +1,7 @@
 """The native argument unpacking: what is not plain goes through ctypes, which accepts or refuses."""
 import ctypes
+import sys
+import types
 
 import pytest
 import torch
@@ -18,6 +20,40 @@ def test_what_is_not_plain_is_left_to_ctypes():
         assert fast.layer_forward(*args) is NotImplemented, (i, odd)
     with pytest.raises(TypeError):
         fast.layer_forward(h)
+
+
+@pytest.mark.parametrize("module", [None, types.SimpleNamespace(TORCH_VERSION="1.0.0")])
+def test_without_a_module_for_this_torch_every_call_goes_through_ctypes(monkeypatch, module):
+    monkeypatch.setitem(sys.modules, B.__package__ + "._fastcall", module)
+    monkeypatch.setattr(B, "_fast", None)
+    with pytest.warns(UserWarning, match="ctypes"):
+        with pytest.raises(B.BlockFFNError) as e:       # the library's own answer to a NULL handle
+            B.blockffn_router(ctypes.c_void_p(0), B.make_weights(), None, 1, None, stream=0)
+    assert e.value.code == B.ERR_INVALID_ARG
+    for call in (lambda: B.blockffn_chunk_union(None, None, 1, None, None, None, stream=0),
+                 lambda: B.blockffn_expert_ffn(None, B.make_weights(), None, None, 1, None, None, None, stream=0),
+                 lambda: B.blockffn_expert_ffn_noalloc(B.Config(), B.make_weights(), None, None, 1, None, None, None, stream=0),
+                 lambda: B.blockffn_layer_forward(None, B.make_weights(), None, 1, None, stream=0),
+                 lambda: B.blockffn_layer_forward_scores(None, B.make_weights(), None, None, 1, None, stream=0),
+                 lambda: B.blockffn_read_routing(None, 1, stream=0),
+                 lambda: B.blockffn_reuse_ratio(None, None, 1, None, stream=0)):
+        with pytest.raises(B.BlockFFNError) as e:
+            call()
+        assert e.value.code == B.ERR_INVALID_ARG
+
+
+@pytest.mark.gpu
+def test_a_layer_without_the_module(monkeypatch):
+    layer, x = B.Layer(256, 40, 64, L_max=5), torch.randn(5, 256, device="cuda").bfloat16()
+    t = {"W_r": torch.randn(40, 256, device="cuda").bfloat16(), "gain": torch.ones(40, device="cuda"),
+         "U": torch.randn(40, 64, 256, device="cuda").bfloat16(), "D": torch.randn(40, 256, 64, device="cuda").bfloat16()}
+    dw = B.DeviceWeights(B.make_weights(t["W_r"], t["gain"], None, t["U"], t["D"]), t)
+    want = layer.forward(dw, x)
+    monkeypatch.setitem(sys.modules, B.__package__ + "._fastcall", None)
+    monkeypatch.setattr(B, "_fast", None)
+    with pytest.warns(UserWarning, match="ctypes"):
+        got = layer.forward(dw, x)
+    assert all(torch.equal(a, b) for a, b in zip(vars(want).values(), vars(got).values()))
 
 
 @pytest.mark.gpu
