@@ -175,19 +175,23 @@ PyObject* routing_buffers(PyObject*, PyObject* const* a, Py_ssize_t n) {
   try {
     const auto dev = at::device(at::Device(at::kCUDA, static_cast<c10::DeviceIndex>(index)));
     const auto i32 = dev.dtype(at::kInt);
-    PyObject* t = PyTuple_New(5);
-    if (!t) return nullptr;
-    auto put = [&](int k, PyObject* o) { PyTuple_SET_ITEM(t, k, o); };
+    at::Tensor b[5];               // (all of them exist before the first becomes a Python object)
     if (with_scores) {
-      put(0, THPVariable_Wrap(at::empty({L, E}, dev.dtype(at::kFloat))));
-      put(1, THPVariable_Wrap(at::empty({L, words}, i32)));
-    } else {
-      put(0, Py_NewRef(Py_None));
-      put(1, Py_NewRef(Py_None));
+      b[0] = at::empty({L, E}, dev.dtype(at::kFloat));
+      b[1] = at::empty({L, words}, i32);
     }
-    put(2, THPVariable_Wrap(at::empty({words}, i32)));
-    put(3, THPVariable_Wrap(at::empty({E}, i32)));
-    put(4, THPVariable_Wrap(at::empty({1}, i32)));
+    b[2] = at::empty({words}, i32);
+    b[3] = at::empty({E}, i32);
+    b[4] = at::empty({1}, i32);
+    PyObject* t = PyTuple_New(5);
+    for (int k = 0; t && k < 5; ++k) {
+      PyObject* o = b[k].defined() ? THPVariable_Wrap(b[k]) : Py_NewRef(Py_None);
+      if (o) {
+        PyTuple_SET_ITEM(t, k, o);
+      } else {
+        Py_CLEAR(t);
+      }
+    }
     return t;
   } catch (const std::exception&) {
     Py_RETURN_NOTIMPLEMENTED;

@@ -22,6 +22,17 @@ def test_what_is_not_plain_is_left_to_ctypes():
         fast.layer_forward(h)
 
 
+def test_buffers_that_cannot_be_allocated_leave_nothing_behind():
+    fast = B._load_fast()
+    args = (1 << 30, 1 << 30, 1 << 30, 0, 1 << 6)      # a device that does not exist
+    for _ in range(3):
+        assert fast.routing_buffers(*args) is NotImplemented
+    before = sys.getallocatedblocks()
+    for _ in range(1000):
+        fast.routing_buffers(*args)
+    assert sys.getallocatedblocks() - before < 500     # (1000 where each call loses its tuple)
+
+
 @pytest.mark.parametrize("module", [None, types.SimpleNamespace(TORCH_VERSION="1.0.0")])
 def test_without_a_module_for_this_torch_every_call_goes_through_ctypes(monkeypatch, module):
     monkeypatch.setitem(sys.modules, B.__package__ + "._fastcall", module)
