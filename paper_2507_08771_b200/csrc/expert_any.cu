@@ -11,9 +11,11 @@
 //                    writes every out[t][c] once (no atomics: results are run-to-run identical).
 //
 // h is kept to 32 bits: it is stored as three bf16 planes that give the fp32 value exactly (24
-// significand bits, cut off 8 at a time; the second and third plane are scaled by 2^8 and 2^16, or
-// they would be denormal, which the tensor cores lose, for h below 1e-35), and the down projection
-// multiplies all three with D.
+// significand bits, cut off 8 at a time), and the down projection multiplies all three with D. The
+// second and third plane are scaled by 2^7 and 2^15, or they would be denormal, which the tensor
+// cores lose, for h below 1e-31. No plane is then larger than the first, so a sum of products with
+// it overflows only where the sum of |h D| does. (An infinite weight gives NaN instead of an
+// infinity where a plane is zero.)
 // Products of bf16 are exact; the sum of 32 of them leaves the tensor core after two mma and is
 // added in fp32 there (a longer chain inside the tensor core would lose bits to its truncation).
 //
@@ -252,11 +254,11 @@ __global__ void __launch_bounds__(kThreads, 2) any_up_kernel(const AnyUpParams p
       const int e = tid + k * kThreads;
       if (at[k] != ~(size_t)0) {
         const float h = sc[k] * swish(sum_warps<NTG>(red, (e >> 4) * kRedTok + (e & 15)));
-        // three bf16, h = h1 + h2 / 2^8 + h3 / 2^16: its significand cut off 8 bits at a time. An
+        // three bf16, h = h1 + h2 / 2^7 + h3 / 2^15: its significand cut off 8 bits at a time. An
         // infinity or NaN has no remainder (and a NaN keeps a bit where the cut would lose it).
         uint32_t h1 = __float_as_uint(h) >> 16, h2 = 0, h3 = 0;
         if ((__float_as_uint(h) & 0x7f800000u) != 0x7f800000u) {
-          const float r = (h - __uint_as_float(h1 << 16)) * 256.0f;
+          const float r = (h - __uint_as_float(h1 << 16)) * 128.0f;
           h2 = __float_as_uint(r) >> 16;
           h3 = __float_as_uint((r - __uint_as_float(h2 << 16)) * 256.0f) >> 16;
         } else if (h != h) {
@@ -396,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, 2) any_down_kernel(const AnyDownPara
 #pragma unroll
     for (int n = 0; n < NTG; ++n)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) hi[n][v] += mid[n][v] * 0x1p-8f + lo[n][v] * 0x1p-16f;
+      for (int v = 0; v < 4; ++v) hi[n][v] += mid[n][v] * 0x1p-7f + lo[n][v] * 0x1p-15f;
     store_tile<NTG>(red + warp * (8 * NTG * kRedTok), hi, g, tg);
     __syncthreads();
 #pragma unroll

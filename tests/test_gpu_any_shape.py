@@ -86,3 +86,21 @@ def test_ends_of_the_float_range():
     assert np.isnan(got[3]).all()
     for t in (0, 1, 2, 4):
         assert np.abs(got[t] - clean[t]).max() <= TOL * np.sqrt(np.mean(clean[t] ** 2))
+
+
+def test_sums_up_to_the_largest_float():
+    """The scaled planes of the intermediate may not overflow in sums that do not. Three neurons give
+    h = 2^126 (1 + 2^-7 - 2^-23), whose second plane is as large as it gets next to the first; the
+    output is their sum, exact to two roundings."""
+    d, E, d_e = 8, 1, 8
+    U, D = torch.zeros(E, d_e, d), torch.zeros(E, d, d_e)
+    U[0, :3, 0], D[0, :, :3] = 32.0, 1.0                   # swish(32) is 32
+    t = {"U": U.bfloat16().cuda(), "D": D.bfloat16().cuda()}
+    h = 2.0 ** 126 * (1 + 2.0 ** -7 - 2.0 ** -23)
+    for L in (1, 9, 17):
+        layer = B.Layer(d, E, d_e, L_max=L, variant=B.VARIANT_SIMT)
+        x = torch.zeros(L, d, dtype=torch.bfloat16, device="cuda")
+        x[:, 0] = 1.0
+        s = torch.full((L, E), h / 32, device="cuda")
+        out = layer.forward_scores(B.DeviceWeights(B.make_weights(U=t["U"], D=t["D"]), t), x, s).out
+        assert ((out.double() - 3 * h).abs() <= 2.0 ** -22 * 3 * h).all()
