@@ -89,7 +89,7 @@ def test_a_token_that_is_not_finite_spoils_only_itself():
     assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
 
 
-def test_wait_that_runs_out_leaves_the_handle_usable():
+def test_wait_that_runs_out_is_reported_every_time():
     d, E, d_e, L = 512, 32, 64, 8
     dw = make(d, E, d_e, 1, -0.5)
     x = torch.randn(L, d, device="cuda").bfloat16()
@@ -99,6 +99,31 @@ def test_wait_that_runs_out_leaves_the_handle_usable():
         held.forward(dw, x, out=out)
         assert held.last_status(clear=True) == B.DEV_WAIT_EXPIRED
         assert bool((out == 7.0).all())
+
+
+@pytest.mark.parametrize("held", [B.CFG_TEST_EXPIRE_WAIT, B.CFG_TEST_EXPIRE_WAIT | B.CFG_NO_SPLIT])
+@pytest.mark.parametrize("L", [4, 12, 24])
+def test_calls_after_one_whose_wait_ran_out(held, L):
+    """One call in the middle of a sequence gives up, at the logits or at h: the
+    next ones find buffers, tickets and marks in order."""
+    d, E, d_e = 512, 40, 64
+    dw, layer = make(d, E, d_e, 7, -0.5), B.Layer(d, E, d_e, L_max=32)
+    cfg = B.Config.from_address(layer.h.value)       # the handle begins with its configuration
+    assert (cfg.d, cfg.E, cfg.d_e, cfg.L_max, cfg.flags) == (d, E, d_e, 32, 0)
+    for k in range(2):                               # (either of the two buffers of h)
+        for n in [L] * (k + 1) + [0] + [L, 32, 1, L]:
+            cfg.flags = 0 if n else held
+            x = torch.randn(n or L, d, device="cuda").bfloat16()
+            out = torch.full((n or L, d), 7.0, device="cuda")
+            B.blockffn_layer_forward(layer.h, dw.struct, x, n or L, out)
+            if n:
+                _, ref = reference(dw.tensors, x)
+                assert layer.last_status() == 0
+                assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+            else:
+                assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+                assert bool((out == 7.0).all())
+    cfg.flags = 0
 
 
 def test_a_new_handle_has_its_workspace_filled():
@@ -119,3 +144,67 @@ def test_a_new_handle_has_its_workspace_filled():
         torch.cuda.synchronize()
     assert layer.last_status() == 0
     assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+
+
+def layers(E=40, d=1024, d_e=64):
+    """Parameters whose layers, one after the other, activate some, few, most, all or none of the experts."""
+    dws = [make(d, E, d_e, s, b) for s, b in enumerate((-0.5, -1.6, 0.8, 9.0, -9.0))]
+    for dw in dws:
+        dw.tensors["D"].mul_(1.0 / E)                # (the running state keeps its scale)
+    return dws
+
+
+def chain(layer, dws, lengths, h, x, flags, each=lambda i: None):
+    for i, L in enumerate(lengths):
+        B.blockffn_layer_forward(layer.h, dws[i % len(dws)].struct, x[i % 2], L, h, x[(i + 1) % 2], None,
+                                 flags | B.CALL_ACCUMULATE)
+        each(i)
+
+
+@pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
+@pytest.mark.parametrize("lengths", [[1], [8], [13], [16], [32], [1, 32, 8, 17, 9, 24, 3, 16]], ids=str)
+@pytest.mark.parametrize("d,E", [(1024, 40), (2048, 64)])
+def test_calls_one_behind_the_other(flags, lengths, d, E):
+    """Nothing but layer calls on the stream, every x from the call before: early reads, the two
+    buffers of h and what they are reset to, the tags of the words. The same bits as with a pause
+    behind every call, where every layer is compared with float64; eagerly and from a graph."""
+    dws, layer = layers(E, d), B.Layer(d, E, 64, L_max=32)
+    lengths = (lengths * 24)[:24]
+    start = torch.randn(32, d, device="cuda")
+    h, x = start.clone(), torch.zeros(2, 32, d, dtype=torch.bfloat16, device="cuda")
+
+    def reset():
+        h.copy_(start)
+        x.copy_(start.expand(2, 32, d))
+    reset()
+    torch.cuda.synchronize()
+    seen = {"h": h.double()}
+
+    def compare(i):
+        L = lengths[i]
+        torch.cuda.synchronize()
+        _, ref = reference(dws[i % len(dws)].tensors, seen.get("x", x[0])[:L])
+        rms = max(ref.square().mean().sqrt().item(), 1e-6)
+        assert (h[:L].double() - seen["h"][:L] - ref).abs().max().item() <= 2e-2 * rms + 1e-5
+        assert torch.equal(x[(i + 1) % 2][:L], h[:L].bfloat16())
+        seen["h"], seen["x"] = h.double(), x[(i + 1) % 2].clone()
+    chain(layer, dws, lengths, h, x, flags, compare)
+    want = (h.clone(), x.clone())
+
+    for _ in range(3):
+        reset()
+        chain(layer, dws, lengths, h, x, flags)
+        torch.cuda.synchronize()
+        assert torch.equal(h, want[0]) and torch.equal(x, want[1])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        reset()
+        chain(layer, dws, lengths, h, x, flags)
+    for _ in range(5):                               # graphs and eager calls in turn, nothing in between
+        graph.replay()
+    reset()
+    chain(layer, dws, lengths, h, x, flags)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(h, want[0]) and torch.equal(x, want[1])
+    assert layer.last_status() == 0
