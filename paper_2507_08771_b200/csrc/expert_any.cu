@@ -14,8 +14,8 @@
 // significand bits, cut off 8 at a time), and the down projection multiplies all three with D. The
 // second and third plane are scaled by 2^7 and 2^15, or they would be denormal, which the tensor
 // cores lose, for h below 1e-31. No plane is then larger than the first, so a sum of products with
-// it overflows only where the sum of |h D| does. (An infinite weight gives NaN instead of an
-// infinity where a plane is zero.)
+// it overflows only where the sum of |h D| does. Their part is left out where it is no number: an
+// infinite weight times a plane that is zero (a NaN of h or D is in the first plane's part as well).
 // Products of bf16 are exact; the sum of 32 of them leaves the tensor core after two mma and is
 // added in fp32 there (a longer chain inside the tensor core would lose bits to its truncation).
 //
@@ -398,7 +398,10 @@ __global__ void __launch_bounds__(kThreads, 2) any_down_kernel(const AnyDownPara
 #pragma unroll
     for (int n = 0; n < NTG; ++n)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) hi[n][v] += mid[n][v] * 0x1p-7f + lo[n][v] * 0x1p-15f;
+      for (int v = 0; v < 4; ++v) {
+        const float rest = mid[n][v] * 0x1p-7f + lo[n][v] * 0x1p-15f;
+        hi[n][v] += rest == rest ? rest : 0.0f;
+      }
     store_tile<NTG>(red + warp * (8 * NTG * kRedTok), hi, g, tg);
     __syncthreads();
 #pragma unroll

@@ -108,6 +108,23 @@ def test_sums_up_to_the_largest_float():
         assert ((out.double() - 3 * h).abs() <= 2.0 ** -22 * 3 * h).all()
 
 
+def test_infinite_weight():
+    """An infinite weight gives an infinity, as one fp32 product does: h = swish(32) = 32 is a bf16, so
+    the planes behind the first are zero, and zero times an infinity is no number."""
+    d, E, d_e = 8, 1, 8
+    U, D = torch.zeros(E, d_e, d), torch.zeros(E, d, d_e)
+    U[0, 0, 0] = 32.0
+    D[0, :, 0] = torch.tensor([float("inf"), -float("inf")] + 6 * [1.0])
+    t = {"U": U.bfloat16().cuda(), "D": D.bfloat16().cuda()}
+    for L in (1, 9, 17):
+        layer = B.Layer(d, E, d_e, L_max=L, variant=B.VARIANT_SIMT)
+        x = torch.zeros(L, d, dtype=torch.bfloat16, device="cuda")
+        x[:, 0] = 1.0
+        s = torch.ones(L, E, device="cuda")
+        out = layer.forward_scores(B.DeviceWeights(B.make_weights(U=t["U"], D=t["D"]), t), x, s).out
+        assert torch.equal(out, (32.0 * D[0, :, 0]).cuda().expand(L, d))
+
+
 @pytest.mark.parametrize("d,E,d_e,L", [(1000, 40, 96, 8), (2048, 64, 128, 8), (1000, 40, 96, 1), (1000, 40, 96, 24)])
 def test_precision_of_one_call(d, E, d_e, L):
     """One call against float64, without a stack that would round x in between. Products are exact;
