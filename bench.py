@@ -816,7 +816,7 @@ def extras(args, torch, device, peak):
     for L in I.L_SWEEP:
         row = {"L": L}
         for name, variant, form in (("tensor_core", 0, 0), ("tensor_core_pair", 0, B.CFG_TWO_KERNELS),
-                                    ("cuda_core", 1, 0)):
+                                    ("any_shape", 1, 0)):
             wl = Workload(2, L, chunks, variant, device, args.flags | form)
             us = timed(wl) * 1e3 / wl.calls_per_step
             hs = wl.layer.stats_host()

@@ -39,8 +39,9 @@ namespace {
 constexpr int kRedTok = 20;   // floats per token of a 16-row partial tile: stores hit 32 banks
 
 // steps a thread keeps in flight, and 16-byte pieces of a step: rows g and g + 8 of the weights
-// and, per group of 8 tokens, x (up) or the three planes of h (down). Up and down CTAs share an
-// SM: about 100 KB each.
+// and, per group of 8 tokens, x (up) or the three planes of h (down). An up and a down CTA
+// share an SM (104 + 108 KB of its 233 at E = 64 with one token group, 109 + 109 with two, 95 + 136
+// with four, there only up to 96 experts).
 __host__ __device__ constexpr int up_pieces(int ntg) { return 2 + ntg; }
 __host__ __device__ constexpr int up_steps(int ntg) { return ntg == 1 ? 8 : ntg == 2 ? 6 : 3; }
 __host__ __device__ constexpr int down_pieces(int ntg) { return 2 + 3 * ntg; }
@@ -523,8 +524,10 @@ cudaError_t launch_expert_any(blockffn_ctx* c, const blockffn_weights* w, const 
   dn.d_e = cfg.d_e;
   dn.accumulate = (call_flags & BLOCKFFN_CALL_ACCUMULATE) ? 1 : 0;
   // Grids: a CTA per 16 rows / columns, two per SM at most (larger calls go through their tiles
-  // in turn). The union is not known here: a quarter more row tiles than the caller's hint, or
-  // the paper's sparsity, gives (CTAs that find no rows only keep the down kernel's from an SM).
+  // in turn; an SM has no room for two down CTAs of 17 to 32 tokens, so from d = 2376 on some of
+  // them come after the others). The union is not known here: a quarter more row tiles than the
+  // caller's hint, or the paper's sparsity, gives (CTAs that find no rows only keep the down
+  // kernel's from an SM).
   int u_exp = (cfg.flags >> 17) & 0x7ff;
   if (u_exp == 0) u_exp = (L == 1 ? cfg.E + 4 : 3 * cfg.E + 5) / (L == 1 ? 8 : 10);
   u_exp += u_exp / 4 + 1;

@@ -16,9 +16,9 @@ pytestmark = pytest.mark.gpu
 
 TOL = 2e-2          # max|err| <= TOL * RMS(ref)
 FLIP_BAND = 1e-3    # |pre-ReLU logit| below which a mask flip is excused
-# (kernel family, config flags): CUDA-core; tensor-core chained (one kernel per call for chunks
-# of at most 8 tokens, the up/down pair for longer ones); the same fully serialised; the pair
-# for every chunk length
+# (kernel family, config flags): any shape, 32-bit intermediate; the staged tensor-core kernels
+# chained (one kernel per call where the call's promises allow it, the up/down pair elsewhere); the
+# same fully serialised; the pair for every call
 VARIANTS = [(B.VARIANT_SIMT, 0), (B.VARIANT_AUTO, 0), (B.VARIANT_AUTO, B.CFG_NO_CHAINING),
             (B.VARIANT_AUTO, B.CFG_TWO_KERNELS)]
 # call flags worth running a tensor-core case under: a dependent call (whole device), weights

@@ -5,7 +5,7 @@ workspace with cudaMalloc: a plug-in inside a host application that has given al
 memory to its own pool, or a latency-critical loop in which allocator calls are forbidden.
 The entry point they get instead keeps its intermediate in a fixed array inside the library.
 This file checks, through the C ABI, that it returns what blockffn_expert_ffn returns
-(CUDA-core variant, so the comparison is exact as well as within the usual tolerance), on two
+(any-shape variant, so the comparison is exact as well as within the usual tolerance), on two
 calls in a row with different inputs (the array keeps the previous call's contents), and that
 it refuses a call whose intermediate would not fit.
 
