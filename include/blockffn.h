@@ -34,7 +34,8 @@
  *     within a second gives up (BLOCKFFN_DEV_WAIT_EXPIRED). A program that shares the GPU with
  *     kernels that hold SMs for that long, or that runs several handles' calls at the same time
  *     on streams of different priorities, sets BLOCKFFN_CFG_TWO_KERNELS: no kernel then waits
- *     for another CTA. Scores-in and list calls without a promise never do.
+ *     for another CTA. Scores-in and list calls without a promise do not have that condition: of
+ *     more than 8 tokens they are launched cooperatively, i.e. start when all their CTAs fit.
  *   - Limits: 1 <= L <= L_max <= 32 per call; d % 8 == 0; d_e % 8 == 0;
  *     1 <= E <= 1024.
  */
@@ -98,8 +99,7 @@ typedef struct {
  * weights while the kernel enqueued before it on the stream is still finishing
  * (programmatic dependent launch); this bit launches them fully serialised instead. */
 #define BLOCKFFN_CFG_NO_CHAINING 0x10000
-/* A call whose x is stable, a router-on layer call and a promised chunk of more than 8 tokens
- * normally run as one kernel whose CTAs exchange the intermediate (and the router's logits); this
+/* A call whose x is stable, a router-on layer call and a chunk of more than 8 tokens normally run as one kernel whose CTAs exchange the intermediate (and the router's logits); this
  * bit selects kernels that follow one another instead (router, up projection, down projection)
  * for all of them. Same results within the tolerance. For programs that share the GPU, see the
  * conventions above, and for comparison.                                                    */
@@ -208,13 +208,17 @@ BLOCKFFN_API blockffn_status blockffn_expert_ffn(blockffn_handle h, const blockf
 /* Whole layer, router on: Eq. 3 -> Union(x) -> Eq. 1/2, everything device side.
  * The scores, masks, ids and count land in the handle's workspace
  * (blockffn_read_routing). stats may be NULL.
- * call_flags: ACCUMULATE as above. With INDEPENDENT_X (x and the weights are stable, see the
- * flag) the router is launched on the handle's own stream, ordered behind layer calls made a
- * few calls earlier on `stream` and in front of this call's expert kernels (event record /
- * wait, also inside a stream capture), so that it runs under the calls before it; the expert
- * kernels then fetch their weights under the previous call as a scores-in call does. The
- * first such calls on a stream, or after the stream or its capture changed, keep the router
- * on `stream`. All work of the call is complete when `stream` has reached its end.        */
+ * call_flags: ACCUMULATE as above. For shapes the one-kernel forms take (d % 64, d <= 2048, d_e a
+ * power of two >= 64, room for the score matrix) the call is one kernel, router included: with INDEPENDENT_X (x and the
+ * weights are stable, see the flag) it overlaps its neighbours, without it waits for the work
+ * before it ahead of its first look at x. Other shapes, and handles with
+ * BLOCKFFN_CFG_TWO_KERNELS, take a router kernel and the two expert kernels. Where the tensor-core
+ * pair takes the shape and INDEPENDENT_X is given, that router is launched on a stream of the
+ * handle's own, ordered behind layer calls made a few calls earlier on `stream` and in front of
+ * this call's expert kernels (event record / wait, also inside a stream capture), so that it runs
+ * under the calls before it; the first such calls on a stream, or after the stream or its capture
+ * changed, keep the router on `stream`. All work of the call is complete when `stream` has reached
+ * its end.                                                                                */
 BLOCKFFN_API blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights* w,
                                                     const void* x, int32_t L, float* out,
                                                     void* x_next, blockffn_stats* stats,

@@ -31,19 +31,23 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
   // The one-kernel form pays off where calls overlap freely, i.e. where x is stable (for a
   // router-on call: the router has finished before the expert stage starts). A call of up to 8
   // tokens in a dependent chain (x comes from the call before) runs as the pair, whose two
-  // hand-overs are shorter than a grid-wide exchange inside one kernel; a longer chunk in such a
-  // chain (weights and scores promised stable) takes the one-kernel form on the whole device,
-  // which keeps its weights in shared memory for all tokens at once. Without a promise it stays
-  // with the pair: the one kernel needs all its CTAs resident at once, and a call that promises
-  // nothing is not to depend on what other streams run (24 tokens, d = 2048, E = 64, union 19, list
-  // given: 15.4 us as the pair, 14.0 as one kernel; 16 tokens 11.2 and 11.6; 32 tokens 18.8 and 14.7).
+  // hand-overs are shorter than a grid-wide exchange inside one kernel; a longer chunk takes the
+  // one-kernel form on the whole device, which reads its weights once for all tokens, where the
+  // pair reads what shared memory does not hold once per 8. Without a promise that kernel is
+  // launched cooperatively (launch_expert_lean). List given, nothing promised, us per call of a
+  // captured sequence, pair and one kernel, d = 2048, E = 64, d_e = 128, unions of 19 / 26 / 61: 9 tokens
+  // 10.6 / 21.0 / 44.1 and 10.9 / 14.1 / 27.5, 16 tokens 10.8 / 22.0 / 45.6 and 11.6 / 14.5 / 29.6, 24
+  // tokens 14.3 / 30.4 / 64.5 and 13.7 / 17.7 / 29.5, 32 tokens 17.8 / 38.4 / 83.5 and 14.5 / 18.2 / 31.1.
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
-  const bool dep_long = !x_stable && !logits && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && L > 8;
+  const bool dep_long = !x_stable && !logits && L > 8;
   const bool dep_inside = !x_stable && logits && logits->a0 == nullptr;   // router inside the kernel
   if ((x_stable || dep_long || dep_inside) &&
-      expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr))
-    return launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, pub,
-                              logits, logits_final, st);
+      expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr)) {
+    const cudaError_t e = launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next,
+                                             call_flags, pub, logits, logits_final, st);
+    if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+    cudaGetLastError();          // (a context with fewer SMs than the device: the pair takes the call)
+  }
   return launch_expert_mma(c, w, x, scores, L, union_ids, n_union, out, x_next, call_flags, pub,
                            logits, logits_final, st);
 }

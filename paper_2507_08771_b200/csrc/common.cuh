@@ -114,8 +114,8 @@ cudaError_t launch_expert_any(blockffn_ctx* c, const blockffn_weights* w, const 
                               const int32_t* n_union, float* out, void* x_next, int call_flags,
                               const RoutingOut* pub, const RouterLogits* logits, cudaStream_t st);
 
-// One-kernel form of the tensor-core expert stage for chunks of at most 8 tokens (same
-// arguments as launch_expert_mma below).
+// One-kernel form of the tensor-core expert stage (same arguments as launch_expert_mma below): calls
+// whose x is stable, and chunks of more than 8 tokens.
 bool expert_lean_supported(const blockffn_ctx* c, int L, bool with_logits, bool shared,
                            bool inside = false);
 size_t expert_lean_ws_bytes(const blockffn_config* cfg, int grid);

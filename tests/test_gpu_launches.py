@@ -1,4 +1,4 @@
-"""Which calls run as one kernel, whose CTAs all have to be resident at once, and which do not."""
+"""Which calls run as one kernel, whose CTAs all have to be resident at once, and how those get there."""
 import pytest
 import torch
 
@@ -17,22 +17,72 @@ def launches(layer, call):
 
 
 @pytest.mark.parametrize("L", [1, 8, 9, 16, 17, 32])
-def test_calls_without_a_promise_need_no_resident_grid(L):
-    """Scores or a list given and nothing promised: kernels that follow one another. With the promise
-    a chunk of more than 8 tokens is one kernel."""
+def test_calls_with_and_without_a_promise(L):
+    """Scores or a list given: a chunk of more than 8 tokens is one kernel, with a promise or (launched
+    when all its CTAs fit) without; with CFG_TWO_KERNELS kernels that follow one another."""
     d, E, d_e = 512, 24, 64
-    dw, layer = make(d, E, d_e, 1, 0.0), B.Layer(d, E, d_e, L_max=L)
+    dw = make(d, E, d_e, 1, 0.0)
     x, scores = torch.randn(L, d, device="cuda").bfloat16(), torch.rand(L, E, device="cuda")
     ids, n = torch.arange(E, device="cuda", dtype=torch.int32), torch.full((1,), E, device="cuda", dtype=torch.int32)
     z = torch.einsum("ejd,td->tej", dw.tensors["U"].double(), x.double())
     ref = torch.einsum("tej,ecj->tc", scores.double()[:, :, None] * z * torch.sigmoid(z), dw.tensors["D"].double())
-    for flags, want in ((0, 2), (B.CALL_INDEPENDENT, 1 if L > 8 else 2)):
-        for call in (lambda out: B.blockffn_layer_forward_scores(layer.h, dw.struct, x, scores, L, out, call_flags=flags),
-                     lambda out: B.blockffn_expert_ffn(layer.h, dw.struct, x, scores, L, ids, n, out, call_flags=flags)):
-            out = torch.zeros(L, d, device="cuda")
-            torch.cuda.synchronize()
-            assert launches(layer, lambda: call(out)) == want
-            assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+    for cfg in (0, B.CFG_TWO_KERNELS):
+        layer = B.Layer(d, E, d_e, L_max=L, flags=cfg)
+        for flags in (0, B.CALL_INDEPENDENT):
+            for call in (lambda out: B.blockffn_layer_forward_scores(layer.h, dw.struct, x, scores, L, out, call_flags=flags),
+                         lambda out: B.blockffn_expert_ffn(layer.h, dw.struct, x, scores, L, ids, n, out, call_flags=flags)):
+                out = torch.zeros(L, d, device="cuda")
+                torch.cuda.synchronize()
+                assert launches(layer, lambda: call(out)) == (1 if L > 8 and not cfg else 2)
+                assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+
+
+@pytest.mark.parametrize("L", [16, 32])
+@pytest.mark.parametrize("graph", [False, True])
+def test_calls_without_a_promise_beside_other_streams(L, graph):
+    """Two handles' calls on streams of different priorities beside a stream of large products: every
+    call gets its places on the SMs as a whole, none gives up waiting, and the results are those of
+    the same calls alone."""
+    d, E, d_e, n = 1024, 32, 64, 40
+    dws = [make(d, E, d_e, s, 0.0) for s in range(2)]
+    layers = [B.Layer(d, E, d_e, L_max=L) for _ in range(2)]
+    x = [torch.randn(L, d, device="cuda").bfloat16() for _ in range(2)]
+    scores = [torch.rand(L, E, device="cuda") for _ in range(2)]
+    outs = [[torch.zeros(L, d, device="cuda") for _ in range(n)] for _ in range(2)]
+    a = torch.randn(2048, 2048, device="cuda").bfloat16()
+
+    def calls(k):
+        for i in range(n):
+            B.blockffn_layer_forward_scores(layers[k].h, dws[k].struct, x[k], scores[k], L, outs[k][i])
+
+    want = []
+    for k in range(2):
+        calls(k)
+        torch.cuda.synchronize()
+        want.append(outs[k][0].clone())
+        assert all(torch.equal(o, want[k]) for o in outs[k])
+        for o in outs[k]:
+            o.zero_()
+    streams = [torch.cuda.Stream(priority=p) for p in (0, -1)]
+    graphs = []
+    for k, st in enumerate(streams):
+        if graph:
+            graphs.append(torch.cuda.CUDAGraph())
+            with torch.cuda.graph(graphs[k], stream=st):
+                calls(k)
+    busy = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(busy):
+        for _ in range(30):
+            b = a @ a
+    for k, st in enumerate(streams):
+        with torch.cuda.stream(st):
+            graphs[k].replay() if graph else calls(k)
+    torch.cuda.synchronize()
+    for k in range(2):
+        assert layers[k].last_status() == 0
+        assert all(torch.equal(o, want[k]) for o in outs[k])
+    del b
 
 
 @pytest.mark.parametrize("d,E,L,want", [
