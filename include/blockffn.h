@@ -99,9 +99,10 @@ typedef struct {
  * weights while the kernel enqueued before it on the stream is still finishing
  * (programmatic dependent launch); this bit launches them fully serialised instead. */
 #define BLOCKFFN_CFG_NO_CHAINING 0x10000
-/* A call whose x is stable, a router-on layer call and a chunk of more than 8 tokens normally run as one kernel whose CTAs exchange the intermediate (and the router's logits); this
- * bit selects kernels that follow one another instead (router, up projection, down projection)
- * for all of them. Same results within the tolerance. For programs that share the GPU, see the
+/* A call whose x is stable, a router-on layer call and a chunk of more than 8 tokens normally run
+ * as one kernel whose CTAs exchange the intermediate (and the router's logits); this bit selects
+ * kernels that follow one another instead (router, up projection, down projection) for all of
+ * them. Same results within the tolerance. For programs that share the GPU, see the
  * conventions above, and for comparison.                                                    */
 #define BLOCKFFN_CFG_TWO_KERNELS 0x20000000
 /* The one-kernel form runs a call whose x is promised stable (BLOCKFFN_CALL_INDEPENDENT_X) on
@@ -156,9 +157,7 @@ typedef struct {
                                        blockffn_chunk_union or blockffn_read_routing (the scores of
                                        blockffn_router are stable from the second call after it on).
                                        x and out may still come from the work just
-                                       before. The weight fetch then overlaps the previous kernel
-                                       (a chunk of more than 8 tokens then runs as one kernel that
-                                       waits for that work before it reads x).                      */
+                                       before. The weight fetch then overlaps the previous kernel.   */
 #define BLOCKFFN_CALL_INDEPENDENT_X 4 /* in addition x is stable in the same sense (the chunk does
                                        not consume the previous call's output); implies
                                        BLOCKFFN_CALL_INDEPENDENT. The up projection then runs in full
@@ -209,9 +208,9 @@ BLOCKFFN_API blockffn_status blockffn_expert_ffn(blockffn_handle h, const blockf
  * The scores, masks, ids and count land in the handle's workspace
  * (blockffn_read_routing). stats may be NULL.
  * call_flags: ACCUMULATE as above. For shapes the one-kernel forms take (d % 64, d <= 2048, d_e a
- * power of two >= 64, room for the score matrix) the call is one kernel, router included: with INDEPENDENT_X (x and the
- * weights are stable, see the flag) it overlaps its neighbours, without it waits for the work
- * before it ahead of its first look at x. Other shapes, and handles with
+ * power of two >= 64, room for the score matrix) the call is one kernel, router included: with
+ * INDEPENDENT_X (x and the weights are stable, see the flag) it overlaps its neighbours, without
+ * it waits for the work before it ahead of its first look at x. Other shapes, and handles with
  * BLOCKFFN_CFG_TWO_KERNELS, take a router kernel and the two expert kernels. Where the tensor-core
  * pair takes the shape and INDEPENDENT_X is given, that router is launched on a stream of the
  * handle's own, ordered behind layer calls made a few calls earlier on `stream` and in front of
