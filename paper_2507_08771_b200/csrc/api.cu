@@ -182,7 +182,8 @@ blockffn_status blockffn_create(const blockffn_config* cfg, blockffn_handle* out
     }
   }
   if (expert_any_setup(cfg->L_max) != cudaSuccess || expert_mma_setup(c) != cudaSuccess ||
-      expert_lean_setup(c) != cudaSuccess || expert_chain_setup(c) != cudaSuccess) {
+      expert_lean_setup(c) != cudaSuccess || expert_chain_setup(c) != cudaSuccess ||
+      expert_cluster_setup(c) != cudaSuccess) {
     cudaFree(base);
     delete c;
     return BLOCKFFN_ERR_CUDA;
@@ -305,8 +306,14 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     // calls never writes what their kernels still read.
     const bool x_stable_call = (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
     const RoutingOut pub_in{h->union_mask, h->union_ids, h->n_union, stats, h->scores, h->tok_mask};
-    if (!x_stable_call && expert_chain_supported(h, L)) {
+    if (!x_stable_call && expert_cluster_supported(h, L)) {
       // x from the call before: one kernel made for that chain, router included
+      h->last_layer_waited_first = false;
+      return launch_expert_cluster(h, w, x, L, out, x_next, call_flags, &pub_in, st) == cudaSuccess
+                 ? BLOCKFFN_OK
+                 : BLOCKFFN_ERR_CUDA;
+    }
+    if (!x_stable_call && expert_chain_supported(h, L)) {
       h->last_layer_waited_first = false;
       return launch_expert_chain(h, w, x, L, out, x_next, call_flags, &pub_in, st) == cudaSuccess
                  ? BLOCKFFN_OK

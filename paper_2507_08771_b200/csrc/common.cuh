@@ -48,7 +48,8 @@ struct blockffn_ctx {
   unsigned long long* lean_seq;   // per ring (four of them, 64 words apart): [0] call tickets,
                                   // [1 .. 16] arrival counters of the ring slots, [17 .. 32] those
                                   // of the logit hand-over when the router runs inside the kernel
-  void* chain_ws;       // ticket, logit words and h buffers of the dependent-chain kernel, or NULL
+  void* chain_ws;       // ticket, logit words and h buffers of the dependent-chain kernels, or NULL
+  int clusters;         // clusters of four CTAs the device holds, one CTA per SM (0: not used)
   float* ones;          // [E] of 1.0f: the gain of the router without RMSNorm
   unsigned int* ticket; // last-block-done counters [8]
   uint32_t* status;     // sticky device status word
@@ -130,9 +131,26 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
 bool expert_chain_supported(const blockffn_ctx* c, int L);
 size_t expert_chain_ws_bytes(const blockffn_config* cfg, int sms);
 cudaError_t expert_chain_setup(blockffn_ctx* c);
+// What is in chain_ws: both kernels of dependent calls work on it and count calls in the same way.
+struct ChainWorkspace {
+  unsigned long long* seq;      // tickets, num_sms per call
+  uint32_t* used;               // [2] 16-byte pieces of each h buffer that its last call wrote
+  unsigned long long* logits;   // copies of [L][E] words {logit, call number}
+  size_t logit_copy;            // words from one copy to the next
+  uint16_t* h;                  // two buffers of h_slot elements
+  size_t h_slot;
+};
+ChainWorkspace chain_workspace(const blockffn_ctx* c);
 cudaError_t launch_expert_chain(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
                                 float* out, void* x_next, int call_flags, const RoutingOut* pub,
                                 cudaStream_t st);
+
+// The same for longer chunks, on clusters of four CTAs (expert_cluster.cu).
+bool expert_cluster_supported(const blockffn_ctx* c, int L);
+cudaError_t expert_cluster_setup(blockffn_ctx* c);
+cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
+                                  float* out, void* x_next, int call_flags, const RoutingOut* pub,
+                                  cudaStream_t st);
 
 // Tensor-core / bulk-copy variant of the expert stage. union_ids == NULL: the kernels derive
 // the union from the nonzero pattern of scores and publish it through pub; with logits != NULL

@@ -1,0 +1,44 @@
+"""Router-on layer calls of 17 to 32 tokens (and of 9 to 16 with a large union) behind one another: one
+kernel on clusters of four CTAs. Edges of its K quarters, row tiles and expert groups; references and
+tolerances as in test_gpu_chain."""
+import pytest
+import torch
+
+from paper_2507_08771_b200 import binding as B
+from test_gpu_chain import check, make, reference
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,E,d_e,L", [
+    (256, 8, 64, 32),          # one k block per quarter; fewer blocks of h than quarters
+    (448, 20, 64, 17),         # quarters of one and two blocks
+    (1984, 40, 512, 25),       # rows in several passes, all columns of a cluster but two
+    (2048, 530, 64, 32),       # more groups of 16 experts than clusters, more than 4 mask words
+    (512, 1024, 64, 20),       # the most experts
+    (2048, 128, 128, 13),      # 9 to 16 tokens
+    (1536, 80, 256, 16),
+])
+def test_edges(d, E, d_e, L):
+    layer = B.Layer(d, E, d_e, L_max=32)
+    g = torch.Generator(device="cuda").manual_seed(d + E)
+    for bias in (-2.4, -1.0, 0.3, 9.0):         # a few, some, most, all of the experts
+        dw = make(d, E, d_e, d + E, bias)
+        x = torch.randn(L, d, device="cuda", generator=g).bfloat16()
+        check(layer, dw, x, B.CALL_INDEPENDENT)
+    assert layer.last_status() == 0
+
+
+@pytest.mark.parametrize("L", [20, 32])
+def test_a_token_that_is_not_finite_spoils_only_itself(L):
+    d, E, d_e = 512, 24, 64
+    layer, dw = B.Layer(d, E, d_e, L_max=L), make(d, E, d_e, 3, -0.5)
+    x = torch.randn(L, d, device="cuda").bfloat16()
+    _, ref = reference(dw.tensors, x)
+    x[18, 5] = float("nan")
+    x[3, 400] = float("inf")
+    out = layer.forward(dw, x).out
+    assert bool(out[18].isnan().all()) and not bool(out[3].isfinite().any())
+    keep = [t for t in range(L) if t not in (3, 18)]
+    assert (out[keep].double() - ref[keep]).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+    assert layer.last_status() == 0
