@@ -31,16 +31,22 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
   // The one-kernel form pays off where calls overlap freely, i.e. where x is stable (for a
   // router-on call: the router has finished before the expert stage starts). A call of up to 8
   // tokens in a dependent chain (x comes from the call before) runs as the pair, whose two
-  // hand-overs are shorter than a grid-wide exchange inside one kernel; a longer chunk takes the
-  // one-kernel form on the whole device, which reads its weights once for all tokens, where the
-  // pair reads what shared memory does not hold once per 8. Without a promise that kernel is
-  // launched cooperatively (launch_expert_lean). List given, nothing promised, us per call of a
-  // captured sequence, pair and one kernel, d = 2048, E = 64, d_e = 128, unions of 19 / 26 / 61: 9 tokens
-  // 10.6 / 21.0 / 44.1 and 10.9 / 14.1 / 27.5, 16 tokens 10.8 / 22.0 / 45.6 and 11.6 / 14.5 / 29.6, 24
-  // tokens 14.3 / 30.4 / 64.5 and 13.7 / 17.7 / 29.5, 32 tokens 17.8 / 38.4 / 83.5 and 14.5 / 18.2 / 31.1.
+  // hand-overs are shorter than a grid-wide exchange inside one kernel. A longer chunk is one kernel, which
+  // reads its weights once for all tokens, where the pair reads what shared memory does not hold once per 8:
+  // on clusters where the union is large (expert_cluster_supported has the figures), else the one-kernel form
+  // on the whole device. Without a promise either is launched cooperatively. List given, nothing promised, us
+  // per call of a captured sequence, pair / one-kernel form / clusters, unions of 19 and 61 of 64 experts at
+  // d = 2048, d_e = 128: 24 tokens 14.3 / 14.1 / 12.6 and 64.5 / 29.7 / 24.1, 32 tokens 17.8 / 14.6 / 12.6 and 83.5 /
+  // 31.2 / 24.8; 16 tokens 10.8 / 11.7 / 11.4 and 45.6 / 29.6 / 22.9.
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
   const bool dep_long = !x_stable && !logits && L > 8;
   const bool dep_inside = !x_stable && logits && logits->a0 == nullptr;   // router inside the kernel
+  if (dep_long && expert_cluster_supported(c, L, false)) {
+    const cudaError_t e = launch_expert_cluster(c, w, x, scores, L, union_ids, n_union, out, x_next,
+                                                call_flags, pub, st);
+    if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+    cudaGetLastError();          // (a context with fewer SMs than the device)
+  }
   if ((x_stable || dep_long || dep_inside) &&
       expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr)) {
     const cudaError_t e = launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next,
@@ -306,10 +312,10 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     // calls never writes what their kernels still read.
     const bool x_stable_call = (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
     const RoutingOut pub_in{h->union_mask, h->union_ids, h->n_union, stats, h->scores, h->tok_mask};
-    if (!x_stable_call && expert_cluster_supported(h, L)) {
+    if (!x_stable_call && expert_cluster_supported(h, L, true)) {
       // x from the call before: one kernel made for that chain, router included
       h->last_layer_waited_first = false;
-      return launch_expert_cluster(h, w, x, L, out, x_next, call_flags, &pub_in, st) == cudaSuccess
+      return launch_expert_cluster(h, w, x, nullptr, L, nullptr, nullptr, out, x_next, call_flags, &pub_in, st) == cudaSuccess
                  ? BLOCKFFN_OK
                  : BLOCKFFN_ERR_CUDA;
     }

@@ -145,12 +145,14 @@ cudaError_t launch_expert_chain(blockffn_ctx* c, const blockffn_weights* w, cons
                                 float* out, void* x_next, int call_flags, const RoutingOut* pub,
                                 cudaStream_t st);
 
-// The same for longer chunks, on clusters of four CTAs (expert_cluster.cu).
-bool expert_cluster_supported(const blockffn_ctx* c, int L);
+// The same for longer chunks, on clusters of four CTAs (expert_cluster.cu), with the router inside
+// (scores == NULL) or scores and maybe the union list given.
+bool expert_cluster_supported(const blockffn_ctx* c, int L, bool router);
 cudaError_t expert_cluster_setup(blockffn_ctx* c);
-cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
-                                  float* out, void* x_next, int call_flags, const RoutingOut* pub,
-                                  cudaStream_t st);
+cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x,
+                                  const float* scores, int L, const int32_t* union_ids,
+                                  const int32_t* n_union, float* out, void* x_next, int call_flags,
+                                  const RoutingOut* pub, cudaStream_t st);
 
 // Tensor-core / bulk-copy variant of the expert stage. union_ids == NULL: the kernels derive
 // the union from the nonzero pattern of scores and publish it through pub; with logits != NULL

@@ -1,6 +1,6 @@
-// A whole layer call of 17 to 32 tokens in a dependent chain (x is what the call before left) as one
-// kernel on clusters of four CTAs: router (Eq. 3), Union(x) (Sec. 3.3), up and down projection
-// (Eq. 1, Eq. 2). The steps and the two exchanges over the whole device are those of
+// A layer call of 9 to 32 tokens in a dependent chain (x is what the call before left) as one kernel on
+// clusters of four CTAs: router (Eq. 3), or scores and maybe the union list given, Union(x) (Sec. 3.3), up and
+// down projection (Eq. 1, Eq. 2); chunks of up to 16 tokens where the union is large (cluster_plan). The steps and the two exchanges over the whole device are those of
 // expert_chain.cu (which see); this file is about what 32 tokens cost there: every CTA took in all
 // of x and of h, 128 + 344 KB, next to 290 KB of weights, and 16 warps fed mma.sync from registers,
 // so that a layer was bound by issue slots (22.6 K of its 46 K cycles per scheduler), by L2 -> SM
@@ -47,9 +47,9 @@ struct Dims {
   static constexpr int T = 8 * NTG, NTH = 128 * NTG, W = 4 * NTG;
   static constexpr int TR = T / kCluster;       // tokens a CTA finishes
   static constexpr int QR = TR / 4;             // ... in groups of four
-  static constexpr int RP = NTG == 4 ? 192 : 128;   // rows of U a cluster takes at a time
+  static constexpr int RP = 192;                // rows of U a cluster takes at a time
   static constexpr int kSweep = NTH / 8;        // rows copied by one instruction of all threads
-  static constexpr int kTmem = NTG == 4 ? 128 : 32;
+  static constexpr int kTmem = NTG == 4 ? 128 : 64;     // columns: three accumulators of T
   static constexpr int kHBlock = T * 128;       // a 64-wide k block of h
   static constexpr int kHSlot = 4 * kHBlock;    // h goes through the down projection four blocks at a time
   // receive buffers: partial sums of the logits, [source][token][16 experts] doubles, and of U x, [source][4
@@ -90,10 +90,13 @@ struct ClusterParams {
   const uint16_t* x;       // bf16 [L][d]
   const uint16_t* U;       // bf16 [E][d_e][d]
   const uint16_t* D;       // bf16 [E][d][d_e]
-  const uint16_t* W_r;     // bf16 [E][d]
+  const uint16_t* W_r;     // MODE 3: bf16 [E][d]
   const float* gain;       // f32 [E]
   const float* bias;       // f32 [E] or NULL
   float eps;
+  const float* scores;     // MODE 0, 1: f32 [L][E]
+  const int32_t* ids_in;   // MODE 1: the caller's union list
+  const int32_t* n_in;
   unsigned long long* logits;   // kCopies times [L][E] words {logit, call number}
   size_t logit_copy;       // words from one copy to the next
   uint16_t* h;             // two buffers of h_slot elements, bf16 [q][d_e / 64][L][64]
@@ -238,7 +241,8 @@ __device__ __forceinline__ const void* at16(const void* base, uint32_t idx16) {
 // The threads that copy, add and store are warps 0 .. W - 1; warp W only feeds the tensor core. (A fence
 // between the proxies waits for the issuing thread's own copies in flight, 0.5 us a stage when the
 // copying threads did it; warp W has none.)
-template <int NTG>
+// MODE: 0 scores given, 1 scores and the caller's union list given, 3 the router runs in the kernel.
+template <int NTG, int MODE>
 __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     expert_cluster_kernel(const ClusterParams p, const __grid_constant__ CUtensorMap d_map) {
   using C = Dims<NTG>;
@@ -300,7 +304,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   constexpr int UN = 16 / W, kHitWords = TR / 2;
   const int ngroups = (E + 15) >> 4;
   const int rep = cl / ngroups;
-  const bool routes = rep < p.reps;
+  const bool routes = MODE == 3 && rep < p.reps;
   uint4 wf[UN][2];
   float bias = 0.0f;
   auto load_wr = [&](int grp) {
@@ -315,10 +319,10 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     }
     bias = p.bias && (tid & 15) < rrows ? __ldg(p.bias + e0 + (tid & 15)) : 0.0f;
   };
-  if (routes && warp < W) load_wr(cl - rep * ngroups);
+  if (MODE == 3 && routes && warp < W) load_wr(cl - rep * ngroups);
   float gains[4];                  // of experts lane, lane + 32, ...
 #pragma unroll
-  for (int u = 0; u < 4; ++u) gains[u] = warp < TR && 32 * u + lane < E ? __ldg(p.gain + 32 * u + lane) : 0.0f;
+  for (int u = 0; u < 4; ++u) gains[u] = MODE == 3 && warp < TR && 32 * u + lane < E ? __ldg(p.gain + 32 * u + lane) : 0.0f;
   if (tid < 8) ctl[tid] = 0;
   if (tid == 32) {
     for (int i = 0; i < 5; ++i) mbar_init(bar + 8 * i, 1);
@@ -344,10 +348,8 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
 
-  pdl_wait();
-
-  // ---- x: this CTA's quarter of every token
-  if (warp < W) {
+  // x: this CTA's quarter of every token
+  auto copy_x = [&]() {
     uint4 v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -359,6 +361,10 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
       const int k = tid + NTH * i, t = (k >> 3) & (T - 1), kb = k / (8 * T);
       if (t < L && kb < nkb) sts128(xs + kb * (T * 128) + t * 128 + (((k & 7) ^ (t & 7)) << 4), v[i]);
     }
+  };
+  if constexpr (MODE == 3) {
+    pdl_wait();
+    if (warp < W) copy_x();
   }
   if (tid == 0) {
     const unsigned long long n = ticket / (unsigned)p.sms;
@@ -376,204 +382,218 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   tc_after();
   // (the barriers are set up; relaxed: a release would wait for the router weights)
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  if (tid == 0) mbar_expect(bar_mask, T * (words + 1) * 4);
+  if (MODE == 3 && tid == 0) mbar_expect(bar_mask, T * (words + 1) * 4);
   __syncwarp();
   const uint32_t tmem = *reinterpret_cast<const uint32_t*>(smem + lay.off_bar + kBarBytes - 8);
 
-  // ---- router: logits of the cluster's experts
-  uint32_t phase_logit = 0;
-  bool joined = false;             // whether the cluster's CTAs are known to have set up their barriers
-  for (int grp = cl - rep * ngroups; routes && grp < ngroups; grp += GC) {
-    const int e0 = 16 * grp, rrows = min(16, E - e0);
-    if (phase_logit) {             // (more experts than 16 per cluster)
-      if (warp < W) load_wr(grp);
+  float resid = 0.0f;
+  uint32_t clear_n = 0;            // pieces of the other h buffer to reset
+  auto after_wait = [&]() {
+    if (p.accumulate && has_out) resid = __ldcg(p.out + (size_t)ot * d + c0 + om);
+    clear_n = __ldcg(p.used + (ctl[6] ^ 1));
+  };
+  auto clear_other = [&](uint32_t i, uint32_t n) {     // by n threads of a CTA, i: this one
+    uint4* other = reinterpret_cast<uint4*>(p.h + (size_t)(ctl[6] ^ 1) * p.h_slot);
+    for (i += bx * n; i < clear_n; i += G * n) other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  };
+  uint32_t odd_tokens = 0;         // tokens with a logit that is not finite
+  bool lost = false;
+  int nu;
+  if constexpr (MODE == 3) {
+    // ---- router: logits of the cluster's experts
+    uint32_t phase_logit = 0;
+    bool joined = false;             // whether the cluster's CTAs are known to have set up their barriers
+    for (int grp = cl - rep * ngroups; routes && grp < ngroups; grp += GC) {
+      const int e0 = 16 * grp, rrows = min(16, E - e0);
+      if (phase_logit) {             // (more experts than 16 per cluster)
+        if (warp < W) load_wr(grp);
+        __syncwarp();
+        cluster_arrive();            // the receive buffers of the group before have been read
+        cluster_wait();
+      }
+      if (warp < W) {
+        float f[NTG][4];
+        zero_acc<NTG>(f);
+#pragma unroll
+        for (int i = 0; i < UN; ++i) {
+          const int v = warp * UN + i;
+          if ((v >> 1) < nkb) {
+#pragma unroll
+            for (int n = 0; n < NTG; ++n) {
+              const uint4 xv = lds128(xs + (v >> 1) * (T * 128) + (8 * n + g) * 128 + (((2 * tg + (v & 1)) ^ g) << 4));
+              float c[4] = {0.f, 0.f, 0.f, 0.f};
+              mma_bf16(c, wf[i][0].x, wf[i][1].x, wf[i][0].y, wf[i][1].y, xv.x, xv.y);
+              mma_bf16(c, wf[i][0].z, wf[i][1].z, wf[i][0].w, wf[i][1].w, xv.z, xv.w);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) f[n][q] += c[q];
+            }
+          }
+        }
+        float* o = red + (warp * T + 2 * tg) * 20 + g;
+#pragma unroll
+        for (int n = 0; n < NTG; ++n, o += 8 * 20) {
+          o[0] = f[n][0];
+          o[20] = f[n][1];
+          o[8] = f[n][2];
+          o[28] = f[n][3];
+        }
+      }
+      if (tid == 0) mbar_expect(bar_logit, T * 16 * 8);
+      if (tid == NTH + 32) mbar_expect(bar_hit, kCluster * kHitWords * 4);
+      __syncthreads();
+      if (!joined) cluster_wait();
+      joined = true;
+      if (warp < W) {                // a CTA finishes the logits of its TR tokens
+        const int t = tid >> 4, m = tid & 15, to = t / TR;
+        // (four of the warps' sums of 32 products in 32 bits, the rest in 64)
+        double sum = 0.0;
+#pragma unroll
+        for (int w = 0; w < W; w += 4) {
+          const float* r = red + (w * T + t) * 20 + m;
+          sum += (double)((r[0] + r[T * 20]) + (r[2 * T * 20] + r[3 * T * 20]));
+        }
+        st_async_f64(map_rank(sbase + lay.off_lrecv + (rank * TR * 16 + (tid & (TR * 16 - 1))) * 8, to), sum,
+                     map_rank(bar_logit, to));
+      }
+      if (warp < kHitWords) {
+        mbar_wait(bar_logit, phase_logit & 1);
+        const int t = rank * TR + (tid >> 4), m = tid & 15;
+        float v = 0.0f;
+        if (t < L && m < rrows) {
+          // (in 64 bits: the bias cancels most of the sum of an expert that is just active)
+          const double* in = reinterpret_cast<const double*>(smem + lay.off_lrecv) + tid;
+          constexpr int s = TR * 16;
+          v = (float)(((in[0] + in[s]) + (in[2 * s] + in[3 * s])) + (double)bias);
+          const unsigned long long word = ((unsigned long long)(uint32_t)ctl[7] << 32) | __float_as_uint(v);
+          unsigned long long* o = p.logits + (size_t)t * E + e0 + m;
+          for (int k = rep; k < kCopies; k += p.reps)
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(o + k * p.logit_copy), "l"(word) : "memory");
+        }
+        // which of the experts some token activates, to the cluster
+        const uint32_t up = __ballot_sync(0xffffffffu, v > 0.0f);
+        if (lane < kCluster)
+          st_async_b32(map_rank(sbase + lay.off_hit + (rank * kHitWords + warp) * 4, lane), (up | (up >> 16)) & 0xffffu,
+                       map_rank(bar_hit, lane));
+      }
+      if (warp == W + 1) {
+        // U of those experts is asked for in L2 here, where that is known first; the CTAs that have the same
+        // experts share them out, a piece per thread
+        mbar_wait(bar_hit, phase_logit & 1);
+        uint32_t hit = 0;
+#pragma unroll
+        for (int k = 0; k < kCluster * kHitWords; ++k) hit |= reinterpret_cast<const uint32_t*>(smem + lay.off_hit)[k];
+        if (lane < rrows && ((hit >> lane) & 1u)) {
+          const uint32_t eb = (uint32_t)d * (uint32_t)d_e * 2u;      // bytes of U_e
+          const uint32_t n = p.reps * kCluster, i = rep * kCluster + rank;
+          const uint32_t share = ((eb + n - 1) / n + 127u) & ~127u, from = i * share;
+          const char* src = reinterpret_cast<const char*>(p.U) + (size_t)(e0 + lane) * eb;
+          if (from < eb)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + from), "r"(min(share, eb - from))
+                         : "memory");
+        }
+      }
+      ++phase_logit;
       __syncwarp();
-      cluster_arrive();            // the receive buffers of the group before have been read
-      cluster_wait();
     }
-    if (warp < W) {
-      float f[NTG][4];
-      zero_acc<NTG>(f);
+    if (!joined) cluster_wait();
+    after_wait();                    // (not before: what the router waits for would come behind these)
+    // ---- everybody's logits of this CTA's tokens, as they arrive, and Eq. 3 on them: a warp has a token
+    if (warp < TR) {
+      const int t = rank * TR + warp;
+      const uint32_t tag = (uint32_t)ctl[7] + (p.hold == 1 ? 0x80000000u : 0u);
+      const unsigned long long* words_in = p.logits + (cl & (kCopies - 1)) * p.logit_copy + (size_t)t * E;
+      SpinBound bound;
+      bool dead = false, finite = true;
+      float ss = 0.0f;
+      for (int w0 = 0; w0 < words && t < L && !dead; w0 += 4) {
+        unsigned long long v[4];
+        uint32_t pend = 0;
 #pragma unroll
-      for (int i = 0; i < UN; ++i) {
-        const int v = warp * UN + i;
-        if ((v >> 1) < nkb) {
+        for (int u = 0; u < 4; ++u)
+          if (32 * (w0 + u) + lane < E) pend |= 1u << u;
+        const uint32_t mine = pend;
+        do {
 #pragma unroll
-          for (int n = 0; n < NTG; ++n) {
-            const uint4 xv = lds128(xs + (v >> 1) * (T * 128) + (8 * n + g) * 128 + (((2 * tg + (v & 1)) ^ g) << 4));
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_bf16(c, wf[i][0].x, wf[i][1].x, wf[i][0].y, wf[i][1].y, xv.x, xv.y);
-            mma_bf16(c, wf[i][0].z, wf[i][1].z, wf[i][0].w, wf[i][1].w, xv.z, xv.w);
+          for (int u = 0; u < 4; ++u)
+            if ((pend >> u) & 1u) v[u] = ld_relaxed_u64(words_in + 32 * (w0 + u) + lane);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) f[n][q] += c[q];
+          for (int u = 0; u < 4; ++u)
+            if (((pend >> u) & 1u) && (uint32_t)(v[u] >> 32) == tag) pend &= ~(1u << u);
+          if (!__any_sync(0xffffffffu, pend != 0)) break;
+          dead = __any_sync(0xffffffffu, bound.expired(p));
+        } while (!dead);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if ((mine >> u) & 1u) {
+            const float a = __uint_as_float((uint32_t)v[u]);
+            finite &= ((uint32_t)v[u] & 0x7f800000u) != 0x7f800000u;
+            const float r = a > 0.0f ? a : 0.0f;
+            ss = fmaf(r, r, ss);
+            a_sm[warp * Es + 32 * (w0 + u) + lane] = r;
           }
         }
       }
-      float* o = red + (warp * T + 2 * tg) * 20 + g;
+      finite = __all_sync(0xffffffffu, finite);
 #pragma unroll
-      for (int n = 0; n < NTG; ++n, o += 8 * 20) {
-        o[0] = f[n][0];
-        o[20] = f[n][1];
-        o[8] = f[n][2];
-        o[28] = f[n][3];
-      }
-    }
-    if (tid == 0) mbar_expect(bar_logit, T * 16 * 8);
-    if (tid == NTH + 32) mbar_expect(bar_hit, kCluster * kHitWords * 4);
-    __syncthreads();
-    if (!joined) cluster_wait();
-    joined = true;
-    if (warp < W) {                // a CTA finishes the logits of its TR tokens
-      const int t = tid >> 4, m = tid & 15, to = t / TR;
-      // (four of the warps' sums of 32 products in 32 bits, the rest in 64)
-      double sum = 0.0;
-#pragma unroll
-      for (int w = 0; w < W; w += 4) {
-        const float* r = red + (w * T + t) * 20 + m;
-        sum += (double)((r[0] + r[T * 20]) + (r[2 * T * 20] + r[3 * T * 20]));
-      }
-      st_async_f64(map_rank(sbase + lay.off_lrecv + (rank * TR * 16 + (tid & (TR * 16 - 1))) * 8, to), sum,
-                   map_rank(bar_logit, to));
-    }
-    if (warp < kHitWords) {
-      mbar_wait(bar_logit, phase_logit & 1);
-      const int t = rank * TR + (tid >> 4), m = tid & 15;
-      float v = 0.0f;
-      if (t < L && m < rrows) {
-        // (in 64 bits: the bias cancels most of the sum of an expert that is just active)
-        const double* in = reinterpret_cast<const double*>(smem + lay.off_lrecv) + tid;
-        constexpr int s = TR * 16;
-        v = (float)(((in[0] + in[s]) + (in[2 * s] + in[3 * s])) + (double)bias);
-        const unsigned long long word = ((unsigned long long)(uint32_t)ctl[7] << 32) | __float_as_uint(v);
-        unsigned long long* o = p.logits + (size_t)t * E + e0 + m;
-        for (int k = rep; k < kCopies; k += p.reps)
-          asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(o + k * p.logit_copy), "l"(word) : "memory");
-      }
-      // which of the experts some token activates, to the cluster
-      const uint32_t up = __ballot_sync(0xffffffffu, v > 0.0f);
-      if (lane < kCluster)
-        st_async_b32(map_rank(sbase + lay.off_hit + (rank * kHitWords + warp) * 4, lane), (up | (up >> 16)) & 0xffffu,
-                     map_rank(bar_hit, lane));
-    }
-    if (warp == W + 1) {
-      // U of those experts is asked for in L2 here, where that is known first; the CTAs that have the same
-      // experts share them out, a piece per thread
-      mbar_wait(bar_hit, phase_logit & 1);
-      uint32_t hit = 0;
-#pragma unroll
-      for (int k = 0; k < kCluster * kHitWords; ++k) hit |= reinterpret_cast<const uint32_t*>(smem + lay.off_hit)[k];
-      if (lane < rrows && ((hit >> lane) & 1u)) {
-        const uint32_t eb = (uint32_t)d * (uint32_t)d_e * 2u;      // bytes of U_e
-        const uint32_t n = p.reps * kCluster, i = rep * kCluster + rank;
-        const uint32_t share = ((eb + n - 1) / n + 127u) & ~127u, from = i * share;
-        const char* src = reinterpret_cast<const char*>(p.U) + (size_t)(e0 + lane) * eb;
-        if (from < eb)
-          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + from), "r"(min(share, eb - from))
-                       : "memory");
-      }
-    }
-    ++phase_logit;
-    __syncwarp();
-  }
-  if (!joined) cluster_wait();
-  // (not before: what the router waits for would come behind these)
-  float resid = 0.0f;
-  if (p.accumulate && has_out) resid = __ldcg(p.out + (size_t)ot * d + c0 + om);
-  const uint32_t clear_n = __ldcg(p.used + (ctl[6] ^ 1));      // pieces of the other h buffer to reset
-  // ---- everybody's logits of this CTA's tokens, as they arrive, and Eq. 3 on them: a warp has a token
-  if (warp < TR) {
-    const int t = rank * TR + warp;
-    const uint32_t tag = (uint32_t)ctl[7] + (p.hold == 1 ? 0x80000000u : 0u);
-    const unsigned long long* words_in = p.logits + (cl & (kCopies - 1)) * p.logit_copy + (size_t)t * E;
-    SpinBound bound;
-    bool dead = false, finite = true;
-    float ss = 0.0f;
-    for (int w0 = 0; w0 < words && t < L && !dead; w0 += 4) {
-      unsigned long long v[4];
-      uint32_t pend = 0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (32 * (w0 + u) + lane < E) pend |= 1u << u;
-      const uint32_t mine = pend;
-      do {
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if ((pend >> u) & 1u) v[u] = ld_relaxed_u64(words_in + 32 * (w0 + u) + lane);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (((pend >> u) & 1u) && (uint32_t)(v[u] >> 32) == tag) pend &= ~(1u << u);
-        if (!__any_sync(0xffffffffu, pend != 0)) break;
-        dead = __any_sync(0xffffffffu, bound.expired(p));
-      } while (!dead);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if ((mine >> u) & 1u) {
-          const float a = __uint_as_float((uint32_t)v[u]);
-          finite &= ((uint32_t)v[u] & 0x7f800000u) != 0x7f800000u;
-          const float r = a > 0.0f ? a : 0.0f;
-          ss = fmaf(r, r, ss);
-          a_sm[warp * Es + 32 * (w0 + u) + lane] = r;
+      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      // (a negative eps marks the router without RMSNorm, Sec. 4.2.3; the gain is then all ones)
+      const float r = p.eps < 0.0f ? 1.0f : 1.0f / sqrtf(ss / (float)E + p.eps);
+      // the token's mask, to the four CTAs of the cluster
+      const uint32_t to = map_rank(sbase + lay.off_mask + t * 4, lane & 3), to_bar = map_rank(bar_mask, lane & 3);
+      for (int w = 0; w < words; ++w) {
+        const int e = 32 * w + lane;
+        float s = 0.0f;
+        if (t < L && e < E) {
+          const float gn = w == 0 ? gains[0] : w == 1 ? gains[1] : w == 2 ? gains[2] : w == 3 ? gains[3] : __ldg(p.gain + e);
+          s = gn * a_sm[warp * Es + e] * r;
+          a_sm[warp * Es + e] = s;
         }
+        const uint32_t m = __ballot_sync(0xffffffffu, s != 0.0f);
+        if (lane < kCluster) st_async_b32(to + w * 128, m, to_bar);
       }
+      if (dead && lane == 0) atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
+      if (lane < kCluster) st_async_b32(to + words * 128, (finite ? 0u : 1u) | (dead ? 2u : 0u), to_bar);
+      __syncwarp();
+    } else if (warp < W) {           // the others put the other h buffer back meanwhile
+      clear_other(tid - 32 * TR, NTH - 32 * TR);
     }
-    finite = __all_sync(0xffffffffu, finite);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    // (a negative eps marks the router without RMSNorm, Sec. 4.2.3; the gain is then all ones)
-    const float r = p.eps < 0.0f ? 1.0f : 1.0f / sqrtf(ss / (float)E + p.eps);
-    // the token's mask, to the four CTAs of the cluster
-    const uint32_t to = map_rank(sbase + lay.off_mask + t * 4, lane & 3), to_bar = map_rank(bar_mask, lane & 3);
-    for (int w = 0; w < words; ++w) {
-      const int e = 32 * w + lane;
-      float s = 0.0f;
-      if (t < L && e < E) {
-        const float gn = w == 0 ? gains[0] : w == 1 ? gains[1] : w == 2 ? gains[2] : w == 3 ? gains[3] : __ldg(p.gain + e);
-        s = gn * a_sm[warp * Es + e] * r;
-        a_sm[warp * Es + e] = s;
-      }
-      const uint32_t m = __ballot_sync(0xffffffffu, s != 0.0f);
-      if (lane < kCluster) st_async_b32(to + w * 128, m, to_bar);
-    }
-    if (dead && lane == 0) atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
-    if (lane < kCluster) st_async_b32(to + words * 128, (finite ? 0u : 1u) | (dead ? 2u : 0u), to_bar);
-    __syncwarp();
-  } else if (warp < W) {           // the others put the other h buffer back meanwhile
-    uint4* other = reinterpret_cast<uint4*>(p.h + (size_t)(ctl[6] ^ 1) * p.h_slot);
-    for (uint32_t i = bx * (NTH - 32 * TR) + tid - 32 * TR; i < clear_n; i += G * (NTH - 32 * TR))
-      other[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    // (twice the limit: a mate whose wait for the logits runs out still says so)
+    mbar_wait(bar_mask, 0, 2);
+    const uint32_t flag = lane < T ? tm[words * 32 + lane] : 0u;
+    odd_tokens = __ballot_sync(0xffffffffu, flag & 1u);      // with a logit that is not finite
+    // A wait that ran out: out is invalid (this cluster's part is not written). The cluster goes through the
+    // rest with an empty union, so that none of its CTAs is left at a barrier.
+    if (__any_sync(0xffffffffu, flag & 2u) && lane == 0) ctl[5] = 1;
+    __syncthreads();
+    lost = ctl[5] != 0;                  // (the same for all threads)
+    nu = union_of_masks(tm, L, words, ids_sm, ctl);
+    if (lost) nu = 0;
+  } else {
+    nu = derive_union<MODE>(p.scores, RouterLogits{}, p.ids_in, p.n_in, L, E, ids_sm, ctl, tm);
+    cluster_wait();
   }
-  // (twice the limit: a mate whose wait for the logits runs out still says so)
-  mbar_wait(bar_mask, 0, 2);
-  const uint32_t flag = lane < T ? tm[words * 32 + lane] : 0u;
-  const uint32_t odd_tokens = __ballot_sync(0xffffffffu, flag & 1u);      // with a logit that is not finite
-  // A wait that ran out: out is invalid (this cluster's part is not written). The cluster goes through the
-  // rest with an empty union, so that none of its CTAs is left at a barrier.
-  if (__any_sync(0xffffffffu, flag & 2u) && lane == 0) ctl[5] = 1;
-  __syncthreads();
-  const bool lost = ctl[5] != 0;       // (the same for all threads)
-  int nu = union_of_masks(tm, L, words, ids_sm, ctl);
-  if (lost) nu = 0;
 
   // ---- the cluster's rows of U: [r0, r0 + nrows) of the union's u * d_e, in fours, RP at a time ------
   const int R = nu * d_e;
   const int rq = (int)__umulhi((unsigned)R >> 2, p.magic_g), rrem = (R >> 2) - rq * GC;
   const int r0 = 4 * (cl * rq + min(cl, rrem)), nrows = 4 * (rq + (cl < rrem ? 1 : 0));
-  const int rmax = min(RP, 4 * (rq + 1));                      // rows of a pass, the same in every pass
+  // rows of a pass: evenly, the same in every cluster
+  const int npass_max = (4 * (rq + 1) + RP - 1) / RP, rmax = 4 * ((rq + npass_max) / npass_max);
   const int slot_bytes = ((rmax + 7) & ~7) * 128;
   const int S = min(kSlots, p.ring / slot_bytes);
-  const int npass = (nrows + RP - 1) / RP;
+  const int npass = (nrows + rmax - 1) / rmax;
   const int pshift = sh - 6;
   // D: 64-wide blocks, this CTA's quarter b0 .. b0 + nb of the union's nu * d_e / 64, four at a time
   const int nblk = nu << pshift, b0 = (nblk * rank) >> 2, nb = ((nblk * (rank + 1)) >> 2) - b0;
   const int nsw = (nb + 3) >> 2, npairs = d_e >> 6;
   const int SD = min(kSlots, lay.off_x / kDSlot), SH = min(kSlots, (lay.off_bar - lay.off_x) / C::kHSlot);
-  const uint32_t acc = tmem + (NTG == 4 ? 2 * T : T);
+  const uint32_t acc = tmem + 2 * T;
 
   if (warp == W) {
     // ======== the warp that feeds the tensor core ========
     int slot = 0, round = 0;
     for (int ps = 0; ps < npass; ++ps) {
-      const int nr = min(RP, nrows - ps * RP);
+      const int nr = min(rmax, nrows - ps * rmax);
       for (int kb = 0; kb < nkb; ++kb) {
         mbar_wait(full + 8 * slot, round & 1);
         fence_async();
@@ -675,10 +695,18 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         if (lane == 0) tok_sm[q] = m;
       }
     };
+    auto rest_of_inputs = [&]() {  // MODE 0, 1: what the work before may have written, and the scores of this CTA's tokens
+      pdl_wait();
+      copy_x();
+      after_wait();
+      if (warp < TR && rank * TR + warp < L)
+        for (int e = lane; e < E; e += 32) a_sm[warp * Es + e] = __ldcg(p.scores + (size_t)(rank * TR + warp) * E + e);
+      copy_sync();
+    };
     int slot = 0, round = 0;       // of the next stage to wait for
     int islot = 0, iround = 0;     // of the next stage to ask for
     for (int ps = 0; ps < npass; ++ps) {
-      const int ra = r0 + ps * RP, nr = min(RP, nrows - ps * RP);
+      const int ra = r0 + ps * rmax, nr = min(rmax, nrows - ps * rmax);
       uint32_t roff[kCopy];        // this thread's rows, in 16-byte units from U
 #pragma unroll
       for (int i = 0; i < kCopy; ++i) {
@@ -696,24 +724,31 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         }
       };
       if (tid == 0) mbar_expect(bar_up, nr * T * 4);
-      if (ps == 0) mark_tokens();
+      if (MODE == 3 && ps == 0) mark_tokens();
       // A stage is handed on when it has landed, `lag` stages (64 to 80 KB) behind the one asked for.
       const int lag = max(1, min(S - 1, kLagBytes / slot_bytes));
-      for (int kb = 0; kb < nkb + lag; ++kb) {
-        if (kb < nkb) {
-          if (kb >= S) mbar_wait(freed + 8 * islot, (iround - 1) & 1);
-          issue_u(kb);
+      int asked = 0;
+      auto ask = [&]() {
+        if (asked < nkb) {
+          if (asked >= S) mbar_wait(freed + 8 * islot, (iround - 1) & 1);
+          issue_u(asked);
         }
         cp_async_commit();
-        if (kb >= lag) {
-          cp_async_wait_newest(lag);
-          __syncwarp();
-          if (lane == 0) mbar_arrive(full + 8 * slot);
-          if (kb + 1 == nkb + lag) mbar_wait(freed + 8 * slot, round & 1);
-          if (++slot == S) {
-            slot = 0;
-            ++round;
-          }
+        ++asked;
+      };
+      if (MODE != 3 && ps == 0) {  // U is on its way before the call before has left x
+        while (asked <= lag) ask();
+        rest_of_inputs();
+      }
+      for (int kb = 0; kb < nkb; ++kb) {
+        while (asked <= kb + lag) ask();
+        cp_async_wait_newest(lag);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full + 8 * slot);
+        if (kb + 1 == nkb) mbar_wait(freed + 8 * slot, round & 1);
+        if (++slot == S) {
+          slot = 0;
+          ++round;
         }
       }
       tc_after();
@@ -784,7 +819,9 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         cluster_wait();
       }
     }
-    if (npass == 0) mark_tokens();
+    if (MODE == 3 && npass == 0) mark_tokens();
+    if (MODE != 3 && npass == 0) rest_of_inputs();
+    if (MODE != 3) clear_other(tid, NTH);
     if (tid == 0) mbar_expect(bar_out, ncols * T * 4);
     copy_sync();
 
@@ -792,7 +829,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     // Four blocks at a time; a thread fetches 32 bytes of h of one block and token, until nothing there is
     // unwritten. (A token that does not activate an expert has zeros there, which need not be fetched,
     // unless a logit of the token is no finite number: then its x may not be either, and zero times that
-    // is a NaN.)
+    // is a NaN. Where the scores are given nothing is known about x, and all of h is fetched.)
     constexpr int kHS = NTG == 4 ? 6 : 4;
     const int hj = tid / (4 * T), ht = (tid >> 2) & (T - 1), hp = tid & 3;
     bool dead = false;
@@ -807,7 +844,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
       for (int k = 0; k < kHS; ++k) {
         const int i = 4 * (base + k) + hj;
         f[k].lo = f[k].hi = make_uint4(0, 0, 0, 0);
-        if (i < nb && ht < L && ((tok_sm[(b0 + i) >> pshift] >> ht) & 1u)) pend |= 1u << k;
+        if (i < nb && ht < L && (MODE != 3 || ((tok_sm[(b0 + i) >> pshift] >> ht) & 1u))) pend |= 1u << k;
       }
       auto look = [&](int n) {
 #pragma unroll
@@ -853,7 +890,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
       if (lane == 0) atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
     }
     // routing results, spread over clusters: a CTA has its tokens' scores
-    if (!lost) {
+    if (MODE == 3 && !lost) {
       for (int i = GC - 1 - cl; i < TR; i += GC) {
         const int t = rank * TR + i;
         for (int w = warp; w < words && t < L; w += W) {
@@ -897,7 +934,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     }
     if (bx == 0 && tid == 0) p.used[ctl[6]] = lost ? (uint32_t)(p.h_slot >> 3) : (uint32_t)((R * L) >> 3);
     if (!lost && rank == 0 && cl == max(GC - 1 - TR, 0)) {
-      // (by the copying warps only: blockDim.x apart, which is more than they are)
+      if (MODE == 1 && tid == 0 && ctl[3]) atomicOr(p.status, (uint32_t)ctl[3]);
       for (int e = tid; e < E; e += NTH) {
         if (p.pub.union_ids) p.pub.union_ids[e] = e < nu ? ids_sm[e] : -1;
         if (p.pub.union_mask && e < words) p.pub.union_mask[e] = (uint32_t)ctl[8 + e];
@@ -950,18 +987,24 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
   pl.ok = true;
   return pl;
 }
-// Chunks of 9 to 16 tokens come here from an expected union of 7 million elements of U on (14 MB): below,
-// the three hops through distributed shared memory cost more than the smaller broadcast saves. us per
-// layer, expert_chain.cu and this kernel: 16 tokens, d = 2048, E = 128, d_e = 128 (union 41, 10.7 M
-// elements) 22.1 and 20.3; 12 tokens, E = 64, d_e = 256 (20, 10.7 M) 22.3 and 20.9; E = 64, d_e = 128 (20,
-// 5.4 M) 16 tokens 13.6 and 13.3, 9 tokens 13.0 and 13.1; 12 tokens, d = 1024, d_e = 64 8.9 and 11.1.
-ClusterPlan cluster_plan(const blockffn_ctx* c, int L) {
-  if (L > 16 && L <= 32) return cluster_plan_of<4>(c->cfg, L, c->clusters);
-  if (L > 8 && L <= 16) {
-    int u_exp = (c->cfg.flags >> 17) & 0x7ff;
-    if (u_exp == 0) u_exp = (3 * c->cfg.E + 5) / 10;
-    if ((long long)u_exp * c->cfg.d_e * c->cfg.d >= 7000000) return cluster_plan_of<2>(c->cfg, L, c->clusters);
-  }
+// Where a call comes here. The hops through distributed shared memory cost a few microseconds that the smaller
+// broadcast and the one pass over the weights have to save, so the line lies at the number of elements of the
+// expected union's U. us per layer of a captured stack, kernel of before / this one (M elements):
+//   router on, 17 to 32 tokens: always. 32 tokens, d = 512, E = 32, d_e = 64 (0.3 M) 11.5 / 11.1; 17 tokens,
+//     d = 1536, E = 48, d_e = 128 (2.8 M) 14.4 / 13.5; 32 tokens, d = 2048, E = 128, d_e = 128 (10 M) 24.8 / 18.3
+//   router on, 9 to 16: from 6 M. 13 tokens, d = 1792, E = 56, d_e = 128 (3.9 M) 11.9 / 12.6; d = 2048, E = 64
+//     (5 M) 12 tokens 13.2 / 13.4, 16 tokens 13.7 / 13.5; E = 96 (7.6 M), 10 tokens 18.4 / 15.7; E = 128 (10 M),
+//     16 tokens 22.2 / 18.1
+//   scores given, 17 to 32: from 4 M. d = 1536, E = 48 (2.9 M), 18 tokens 11.3 / 11.7; d = 2048, E = 100,
+//     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 64, d_e = 128 (5 M), 24 tokens 15.7 / 13.7; E = 128 (10 M),
+//     32 tokens 24.2 / 17.2
+//   scores given, 9 to 16: from 6 M. d = 2048, E = 64 (5 M) 8.8 / 8.7; E = 128 (10 M), 16 tokens 19.5 / 15.6
+ClusterPlan cluster_plan(const blockffn_ctx* c, int L, bool router) {
+  int u_exp = (c->cfg.flags >> 17) & 0x7ff;
+  if (u_exp == 0) u_exp = (3 * c->cfg.E + 5) / 10;
+  const long long u = (long long)u_exp * c->cfg.d_e * c->cfg.d;
+  if (L > 16 && L <= 32 && (router || u >= 4000000)) return cluster_plan_of<4>(c->cfg, L, c->clusters);
+  if (L > 8 && L <= 16 && u >= 6000000) return cluster_plan_of<2>(c->cfg, L, c->clusters);
   return ClusterPlan{};
 }
 
@@ -993,9 +1036,9 @@ TensorMapEncoder tensor_map_encoder() {
   }();
   return f;
 }
-template <int NTG>
+template <int NTG, int MODE>
 cudaError_t cluster_attr() {
-  const void* f = reinterpret_cast<const void*>(&expert_cluster_kernel<NTG>);
+  const void* f = reinterpret_cast<const void*>(&expert_cluster_kernel<NTG, MODE>);
   cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1004,23 +1047,27 @@ cudaError_t cluster_attr() {
 
 }  // namespace
 
-bool expert_cluster_supported(const blockffn_ctx* c, int L) {
+bool expert_cluster_supported(const blockffn_ctx* c, int L, bool router) {
   if (c->chain_ws == nullptr || (c->cfg.flags & BLOCKFFN_CFG_TWO_KERNELS)) return false;
-  return cluster_plan(c, L).ok;
+  return cluster_plan(c, L, router).ok;
 }
 
 // How many clusters fit the device at one CTA per SM (0: none do, or no chunk length takes them).
 cudaError_t expert_cluster_setup(blockffn_ctx* c) {
   c->clusters = 0;
   if (!c->chain_ws || c->cfg.L_max <= 8 || !tensor_map_encoder()) return cudaSuccess;
-  cudaError_t e = cluster_attr<4>();
-  if (e == cudaSuccess) e = cluster_attr<2>();
+  cudaError_t e = cluster_attr<4, 3>();
+  if (e == cudaSuccess) e = cluster_attr<4, 0>();
+  if (e == cudaSuccess) e = cluster_attr<4, 1>();
+  if (e == cudaSuccess) e = cluster_attr<2, 3>();
+  if (e == cudaSuccess) e = cluster_attr<2, 0>();
+  if (e == cudaSuccess) e = cluster_attr<2, 1>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t lc{};
   cudaLaunchAttribute attr[2];
   cluster_config(lc, attr, c->num_sms / kCluster, Dims<4>::NTH + 64, kSmemMax);
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(&expert_cluster_kernel<4>), &lc) !=
+  if (cudaOccupancyMaxActiveClusters(&n, reinterpret_cast<const void*>(&expert_cluster_kernel<4, 3>), &lc) !=
       cudaSuccess) {
     cudaGetLastError();
     return cudaSuccess;
@@ -1029,19 +1076,24 @@ cudaError_t expert_cluster_setup(blockffn_ctx* c) {
   return cudaSuccess;
 }
 
-cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
-                                  float* out, void* x_next, int call_flags, const RoutingOut* pub,
-                                  cudaStream_t st) {
-  const ClusterPlan pl = cluster_plan(c, L);
+cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x, const float* scores,
+                                  int L, const int32_t* union_ids, const int32_t* n_union, float* out,
+                                  void* x_next, int call_flags, const RoutingOut* pub, cudaStream_t st) {
+  const ClusterPlan pl = cluster_plan(c, L, scores == nullptr);
   if (!pl.ok || !c->chain_ws) return cudaErrorNotSupported;
   const ChainWorkspace ws = chain_workspace(c);
   ClusterParams p{};
   p.x = static_cast<const uint16_t*>(x);
   p.U = static_cast<const uint16_t*>(w->U);
   p.D = static_cast<const uint16_t*>(w->D);
-  p.W_r = static_cast<const uint16_t*>(w->W_r);
-  p.gain = router_gain(c, w);
-  p.bias = w->bias;
+  if (!scores) {
+    p.W_r = static_cast<const uint16_t*>(w->W_r);
+    p.gain = router_gain(c, w);
+    p.bias = w->bias;
+  }
+  p.scores = scores;
+  p.ids_in = union_ids;
+  p.n_in = n_union;
   p.eps = c->cfg.rms_eps;
   p.seq = ws.seq;
   p.sms = c->num_sms;
@@ -1065,7 +1117,7 @@ cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, co
   p.early = (call_flags & (BLOCKFFN_CALL_INDEPENDENT | BLOCKFFN_CALL_INDEPENDENT_X)) ? 1 : 0;
   const int groups = (c->cfg.E + 15) / 16;
   p.reps = pl.clusters >= groups ? pl.clusters / groups : 1;
-  p.hold = !(c->cfg.flags & BLOCKFFN_CFG_TEST_EXPIRE_WAIT) ? 0 : (c->cfg.flags & BLOCKFFN_CFG_NO_SPLIT) ? 2 : 1;
+  p.hold = !(c->cfg.flags & BLOCKFFN_CFG_TEST_EXPIRE_WAIT) ? 0 : scores || (c->cfg.flags & BLOCKFFN_CFG_NO_SPLIT) ? 2 : 1;
   p.wait_ns = 1000000000ull;      // one second
   p.status = c->status;
   if (pub) p.pub = *pub;
@@ -1074,6 +1126,13 @@ cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, co
   cluster_config(lc, attr, pl.clusters, 128 * pl.ntg + 64, pl.smem);
   lc.stream = st;
   lc.numAttrs = (c->cfg.flags & BLOCKFFN_CFG_NO_CHAINING) ? 1 : 2;
+  if (scores && !p.early) {
+    // A call that promises nothing is not to depend on what other streams run: a cooperative launch starts
+    // when all its CTAs fit, so that none of them waits for one that has no place.
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
+    lc.numAttrs = 2;
+  }
   // D as rows of d_e, copied 64 rows x 64 at a time (rows beyond the last expert's come as zeros)
   CUtensorMap map;
   const cuuint64_t dims[2] = {(cuuint64_t)c->cfg.d_e, (cuuint64_t)c->cfg.E * c->cfg.d};
@@ -1083,8 +1142,13 @@ cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, co
                            steps, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  const cudaError_t e = pl.ntg == 4 ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<4>, p, map)
-                                    : cudaLaunchKernelEx(&lc, expert_cluster_kernel<2>, p, map);
+  const int mode = !scores ? 3 : union_ids ? 1 : 0;
+  const cudaError_t e = pl.ntg == 4 ? mode == 3   ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<4, 3>, p, map)
+                                      : mode == 1 ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<4, 1>, p, map)
+                                                  : cudaLaunchKernelEx(&lc, expert_cluster_kernel<4, 0>, p, map)
+                        : mode == 3   ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<2, 3>, p, map)
+                        : mode == 1   ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<2, 1>, p, map)
+                                      : cudaLaunchKernelEx(&lc, expert_cluster_kernel<2, 0>, p, map);
   if (e == cudaSuccess) c->launches += 1;
   return e;
 }
