@@ -846,29 +846,23 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         f[k].lo = f[k].hi = make_uint4(0, 0, 0, 0);
         if (i < nb && ht < L && (MODE != 3 || ((tok_sm[(b0 + i) >> pshift] >> ht) & 1u))) pend |= 1u << k;
       }
-      auto look = [&](int n) {
+      // (all of them at once: waiting for the first four blocks alone first cost 24 tokens with scores given 4 %)
+      auto look = [&]() {
 #pragma unroll
         for (int k = 0; k < kHS; ++k)
-          if (k < n && ((pend >> k) & 1u)) ld_relaxed_v8(f[k], h_at + k * h_step);
+          if ((pend >> k) & 1u) ld_relaxed_v8(f[k], h_at + k * h_step);
 #pragma unroll
         for (int k = 0; k < kHS; ++k)
-          if (k < n && ((pend >> k) & 1u) && !unwritten(f[k]) && p.hold != 2) pend &= ~(1u << k);
+          if (((pend >> k) & 1u) && !unwritten(f[k]) && p.hold != 2) pend &= ~(1u << k);
       };
-      // (the first four blocks alone until they are there: the others are then, or nearly, and what an SM
-      // takes in is what this phase waits for)
-      look(1);
-      while (!dead && __any_sync(0xffffffffu, pend & 1u)) {
-        dead = __any_sync(0xffffffffu, bound.expired(p));
-        look(1);
-      }
-      look(kHS);
+      look();
 #pragma unroll
       for (int k = 0; k < kHS; ++k) {
         const int s = base + k;
         if (s < nsw) {
           while (!dead && __any_sync(0xffffffffu, (pend >> k) & 1u)) {
             dead = __any_sync(0xffffffffu, bound.expired(p));
-            look(kHS);
+            look();
           }
           if (hround > 0) mbar_wait(freed_h + 8 * hs, (hround - 1) & 1);
           if (4 * s + hj < nb) {
@@ -996,8 +990,8 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
 //     (5 M) 12 tokens 13.2 / 13.4, 16 tokens 13.7 / 13.5; E = 96 (7.6 M), 10 tokens 18.4 / 15.7; E = 128 (10 M),
 //     16 tokens 22.2 / 18.1
 //   scores given, 17 to 32: from 4 M. d = 1536, E = 48 (2.9 M), 18 tokens 11.3 / 11.7; d = 2048, E = 100,
-//     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 64, d_e = 128 (5 M), 24 tokens 15.7 / 13.7; E = 128 (10 M),
-//     32 tokens 24.2 / 17.2
+//     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 64, d_e = 128 (5 M), 24 tokens 15.7 / 13.2; E = 128 (10 M),
+//     32 tokens 24.2 / 16.9
 //   scores given, 9 to 16: from 6 M. d = 2048, E = 64 (5 M) 8.8 / 8.7; E = 128 (10 M), 16 tokens 19.5 / 15.6
 ClusterPlan cluster_plan(const blockffn_ctx* c, int L, bool router) {
   int u_exp = (c->cfg.flags >> 17) & 0x7ff;
