@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   float gains[4];                  // of experts lane, lane + 32, ...
 #pragma unroll
   for (int u = 0; u < 4; ++u) gains[u] = MODE == 3 && warp < TR && 32 * u + lane < E ? __ldg(p.gain + 32 * u + lane) : 0.0f;
-  if (tid < 8) ctl[tid] = 0;
+  if (tid < 6) ctl[tid] = 0;       // ([6], [7]: by thread 0 below, with no barrier in between)
   if (tid == 32) {
     for (int i = 0; i < 5; ++i) mbar_init(bar + 8 * i, 1);
     mbar_init(u_begun, 1);

@@ -84,3 +84,68 @@ def test_scores_given(d, E, d_e, L, flags, listed):
         assert torch.equal(nxt[:rows], out[:rows].bfloat16())
         if nan:
             assert bool(out[L - 1].isnan().all())
+
+
+@pytest.mark.parametrize("listed", [False, True])
+@pytest.mark.parametrize("d,E,d_e,L", [(2048, 128, 128, 12), (2048, 64, 256, 16), (2048, 64, 128, 20), (2048, 128, 128, 32)])
+def test_scores_given_one_behind_the_other(d, E, d_e, L, listed):
+    """Nothing but such calls on the stream, every x from the call before and U asked for under it: call
+    numbers, the two buffers of h, tensor memory of two calls on an SM (up to 16 tokens). The same bits as with
+    a pause behind every call, where every layer is compared with float64; eagerly and from a graph."""
+    n, u = 12, E * 3 // 10
+    g = torch.Generator(device="cuda").manual_seed(L)
+    dws = [make(d, E, d_e, s, 0.0) for s in range(3)]
+    layer = B.Layer(d, E, d_e, L_max=32)
+    scores, ids = [], []
+    for i in range(n):
+        k = (u, E, 1, u)[i % 4]                        # (most experts, one: rows in several passes, few rows)
+        pick = torch.randperm(E, device="cuda", generator=g)[:k].sort().values.int()
+        s = torch.zeros(L, E, device="cuda")
+        s[:, pick.long()] = (torch.rand(L, k, device="cuda", generator=g) < 0.5) * (0.5 / k) + 0.1 / k
+        scores.append(s)
+        ids.append(torch.cat([pick, torch.full((E - k,), -1, dtype=torch.int32, device="cuda")]))
+    counts = [torch.tensor([(u, E, 1, u)[i % 4]], dtype=torch.int32, device="cuda") for i in range(n)]
+    start = torch.randn(L, d, device="cuda", generator=g)
+    h, x = start.clone(), torch.zeros(2, L, d, dtype=torch.bfloat16, device="cuda")
+
+    def chain(each=lambda i: None):
+        h.copy_(start)
+        x.copy_(start.expand(2, L, d))
+        for i in range(n):
+            w, xi, xn = dws[i % 3].struct, x[i % 2], x[(i + 1) % 2]
+            if listed:
+                B.blockffn_expert_ffn(layer.h, w, xi, scores[i], L, ids[i], counts[i], h, xn,
+                                      B.CALL_ACCUMULATE | B.CALL_INDEPENDENT)
+            else:
+                B.blockffn_layer_forward_scores(layer.h, w, xi, scores[i], L, h, xn, None,
+                                                B.CALL_ACCUMULATE | B.CALL_INDEPENDENT)
+            each(i)
+    seen = {"h": start.double(), "x": start.bfloat16()}
+
+    def compare(i):
+        torch.cuda.synchronize()
+        t = dws[i % 3].tensors
+        z = torch.einsum("ejd,td->tej", t["U"].double(), seen["x"].double())
+        ref = torch.einsum("tej,ecj->tc", scores[i].double()[:, :, None] * z * torch.sigmoid(z), t["D"].double())
+        assert (h.double() - seen["h"] - ref).abs().max().item() <= 2e-2 * ref.square().mean().sqrt().item() + 1e-5
+        seen["h"], seen["x"] = h.double(), x[(i + 1) % 2].clone()
+        assert torch.equal(seen["x"], h.bfloat16())
+    torch.cuda.synchronize()
+    before = layer.launch_count()
+    chain(compare)
+    assert layer.launch_count() - before == n          # one kernel each
+    want = (h.clone(), x.clone())
+    for _ in range(3):
+        chain()
+    torch.cuda.synchronize()
+    assert torch.equal(h, want[0]) and torch.equal(x, want[1])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain()
+    for _ in range(5):
+        graph.replay()
+    chain()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(h, want[0]) and torch.equal(x, want[1])
+    assert layer.last_status() == 0
