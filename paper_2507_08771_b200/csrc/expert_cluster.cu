@@ -659,7 +659,12 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
       cluster_arrive();
       cluster_wait();
     }
-    if (npass > 0) mbar_wait(u_done, 0);
+    // (a cluster without rows still copies D: the router's partial sums were there, and no fence for the
+    // tensor core has come between them and these copies)
+    if (npass > 0)
+      mbar_wait(u_done, 0);
+    else
+      fence_async();
     int slot = 0, round = 0;
     for (int s = 0; s < nsw; ++s) {
       if (s >= SD) mbar_wait(freed_d + 8 * slot, (round - 1) & 1);

@@ -29,6 +29,24 @@ def test_edges(d, E, d_e, L):
     assert layer.last_status() == 0
 
 
+@pytest.mark.parametrize("d,E,d_e,L", [(2048, 160, 64, 16), (2048, 64, 64, 32), (256, 8, 64, 17)])
+def test_one_expert_router_on(d, E, d_e, L):
+    """64 rows of U in fours: half of the clusters have none, but columns of D like the others."""
+    layer, dws = B.Layer(d, E, d_e, L_max=L), [make(d, E, d_e, s, -12.0) for s in range(4)]
+    g = torch.Generator(device="cuda").manual_seed(E)
+    for i, dw in enumerate(dws):
+        dw.tensors["bias"][(5 * i) % E] = 12.0
+    x = torch.randn(L, d, device="cuda", generator=g).bfloat16()
+    for dw in dws:
+        check(layer, dw, x, B.CALL_INDEPENDENT)
+    out = torch.zeros(L, d, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(40):
+        B.blockffn_layer_forward(layer.h, dws[i % 4].struct, x, L, out, None, None, B.CALL_INDEPENDENT | B.CALL_ACCUMULATE)
+    ref = 10 * sum(reference(dw.tensors, x)[1] for dw in dws)
+    assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt() and layer.last_status() == 0
+
+
 @pytest.mark.parametrize("L", [20, 32])
 def test_a_token_that_is_not_finite_spoils_only_itself(L):
     d, E, d_e = 512, 24, 64
