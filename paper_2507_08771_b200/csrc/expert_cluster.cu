@@ -588,6 +588,8 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   const int nsw = (nb + 3) >> 2, npairs = d_e >> 6;
   const int SD = min(kSlots, lay.off_x / kDSlot), SH = min(kSlots, (lay.off_bar - lay.off_x) / C::kHSlot);
   const uint32_t acc = tmem + 2 * T;
+  // (what the two warps below wait for comes behind x: their limits must not run while the call before does)
+  if (MODE != 3 && warp >= W) pdl_wait();
 
   if (warp == W) {
     // ======== the warp that feeds the tensor core ========

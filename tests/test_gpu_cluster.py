@@ -167,3 +167,30 @@ def test_scores_given_one_behind_the_other(d, E, d_e, L, listed):
     torch.cuda.synchronize()
     assert torch.equal(h, want[0]) and torch.equal(x, want[1])
     assert layer.last_status() == 0
+
+
+@pytest.mark.parametrize("L", [12, 32])
+def test_a_call_behind_one_that_gives_up(L):
+    """The call before holds the device until its wait has run out. Those of the next one, whose CTAs are
+    there already, start behind it."""
+    d, E, d_e = 2048, 128, 128
+    layer, dw = B.Layer(d, E, d_e, L_max=L), make(d, E, d_e, 1, 0.0)
+    cfg = B.Config.from_address(layer.h.value)       # the handle begins with its configuration
+    assert (cfg.d, cfg.E, cfg.d_e, cfg.L_max, cfg.flags) == (d, E, d_e, L, 0)
+    x = torch.randn(L, d, device="cuda").bfloat16()
+    scores = torch.rand(L, E, device="cuda") * (torch.arange(E, device="cuda") % 3 == 0)
+    want, held, out = (torch.full((L, d), 7.0, device="cuda") for _ in range(3))
+
+    def call(o, flags):
+        cfg.flags = flags
+        B.blockffn_layer_forward_scores(layer.h, dw.struct, x, scores, L, o, call_flags=B.CALL_INDEPENDENT)
+        cfg.flags = 0
+    torch.cuda.synchronize()
+    call(want, 0)
+    for _ in range(3):
+        out.fill_(7.0)
+        torch.cuda.synchronize()
+        call(held, B.CFG_TEST_EXPIRE_WAIT)
+        call(out, 0)
+        assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+        assert bool((held == 7.0).all()) and torch.equal(out, want)
