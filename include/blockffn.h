@@ -115,7 +115,9 @@ typedef struct {
  * after two milliseconds, sets BLOCKFFN_DEV_WAIT_EXPIRED and leaves out untouched. Exercises
  * the bounded wait without any fault. (A dependent router-on call has two such waits: this bit
  * alone holds the first, for the router's logits, with BLOCKFFN_CFG_NO_SPLIT the second, for the
- * intermediate.)                                                                          */
+ * intermediate. Calls on clusters of CTAs: with BLOCKFFN_CFG_NO_CHAINING one CTA alone gives up,
+ * behind the logits or waiting for the intermediate; in the second case the columns of the other
+ * clusters are written.)                                                                  */
 #define BLOCKFFN_CFG_TEST_EXPIRE_WAIT 0x10000000
 /* How many experts the caller expects in a chunk's union (1 .. E), bits 17-27 of flags. The
  * tensor-core kernels size their shared memory before the union is known: when the expected

@@ -14,20 +14,20 @@ __device__ __forceinline__ unsigned long long clock_ns() {
   return t;
 }
 // A bound for a spin: expired() is called once per turn and looks at the clock every 32nd.
-// P: parameters with hold, wait_ns and status; times: how many limits long.
+// P: parameters with hold, wait_ns and status.
 struct SpinBound {
   unsigned long long t0 = 0;
   unsigned n = 0;
   template <class P>
-  __device__ __forceinline__ bool expired(const P& p, unsigned times = 1) {
+  __device__ __forceinline__ bool expired(const P& p) {
     if (++n & 31u) return false;
     const unsigned long long now = clock_ns();
     if (t0 == 0) t0 = now;
     const unsigned long long el = now - t0;
-    if (el > times * (p.hold ? 2000000ull : p.wait_ns)) return true;
+    if (el > (p.hold ? 2000000ull : p.wait_ns)) return true;
     // once a wait has run out on this handle the later ones give up quickly, until the caller has
     // read and cleared the status word
-    return el > times * 1000000ull &&
+    return el > 1000000ull &&
            (*reinterpret_cast<volatile uint32_t*>(p.status) & BLOCKFFN_DEV_WAIT_EXPIRED) != 0;
   }
 };

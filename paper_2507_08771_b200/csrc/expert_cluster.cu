@@ -60,7 +60,7 @@ struct Dims {
 
 constexpr int kSlots = 8;              // of either ring, at most
 constexpr int kLagBytes = 64 * 1024;   // of U on the way (20 KB: 698 us a pass of 36 layers, 48 KB 659, 80 KB 655)
-constexpr int kBarBytes = 512;         // mbarriers: 7 + 6 kSlots; at the end the address of the tensor memory
+constexpr int kBarBytes = 512;         // mbarriers: 10 + 6 kSlots; at the end the address of the tensor memory
 
 struct ClusterLayout {
   int off_x, off_lrecv, off_urecv, off_bar, off_ctl, off_ids, off_tok, off_mask, off_score, off_hit, off_drecv, total;
@@ -113,8 +113,10 @@ struct ClusterParams {
   int accumulate;
   int early;               // the weights are stable: read before the wait
   int reps;                // clusters that compute the logits of the same 16 experts
-  int hold;                // test aid: wait for what never comes, 1 the logits, 2 h
-  unsigned long long wait_ns;
+  int hold;                // test aid: wait for what never comes, 1 the logits, 2 h, 3 and 4 one CTA alone for
+                           // the masks, for h
+  int time_shift;          // ... of waits inside one: two to three times 2^time_shift ns from the call's start
+  unsigned long long wait_ns;   // limit of a wait for other clusters
   uint32_t* status;
   RoutingOut pub;
 };
@@ -134,6 +136,19 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, int parity) {
                : "r"(bar), "r"(parity)
                : "memory");
   return ok != 0;
+}
+// (for what other CTAs' arrivals release)
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, int parity) {
+  uint32_t ok;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+               "selp.b32 %0, 1, 0, p;\n}"
+               : "=r"(ok)
+               : "r"(bar), "r"(parity)
+               : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
   uint32_t a;
@@ -271,21 +286,31 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   const uint32_t full_h = freed_d + 8 * kSlots, freed_h = full_h + 8 * kSlots;       // of h
   const uint32_t u_begun = freed_h + 8 * kSlots, bar_hit = u_begun + 8;
 
-  // waits, bounded, for a phase of an mbarrier; a wait that runs out marks the call as dead
-  auto mbar_wait1 = [&](uint32_t b, int parity, int times = 1) {
-    SpinBound limit;
-    while (!mbar_try(b, parity)) {
-      if (limit.expired(p, times)) {
-        ctl[5] = 1;
-        atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
+  const uint32_t acc_read = bar_hit + 8, recv_read = acc_read + 8;  // sums of a pass read, by this CTA, by the cluster
+  const uint32_t bar_end = recv_read + 8;
+
+  // How a call gives up. Waits for other clusters (logits, h) have a limit; one that runs out is told to the
+  // CTA's mates, with the masks or with the last partial sums, and sets ctl[5]: this CTA writes no out. All go on
+  // as if what was waited for had come, so the mates' waits (mbar_wait, for one another and inside a CTA) end.
+  // Those have one limit for the call, well above the others, in case a mate makes no progress at all. A wait that
+  // passes it sets ctl[4], and all later ones of the CTA are over at once: it sends no sums of U x any more, stores no
+  // h and copies no D. However a call ends, all threads pass the same barriers of the CTA and of the cluster: their
+  // number depends on nothing that was waited for.
+  // (There are some thirty such waits, and code that every warp runs once is short of instruction fetch: with a start
+  // time and the bookkeeping of a wait that ran out in each of them 32 tokens took 690 us a pass of 36 layers, so 668.)
+  auto broken = [&]() { return *reinterpret_cast<const volatile int*>(ctl + 4) != 0; };
+  auto coarse_time = [&]() { return (uint32_t)(clock_ns() >> p.time_shift); };
+  uint32_t deadline = coarse_time() + 3;
+  auto wait_for = [&](auto&& done) {
+    while (!done()) {
+      if ((int)(coarse_time() - deadline) >= 0) {
+        ctl[4] = 1;
         break;
       }
     }
-  };
-  auto mbar_wait = [&](uint32_t b, int parity, int times = 1) {
-    mbar_wait1(b, parity, times);
     __syncwarp();
   };
+  auto mbar_wait = [&](uint32_t b, int parity) { wait_for([&]() { return mbar_try(b, parity); }); };
   auto copy_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(NTH) : "memory"); };   // the copying warps
 
   // Everything that is asked for from memory first (ticket, router weights, then x) is on its way at once.
@@ -328,6 +353,9 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     for (int i = 0; i < 5; ++i) mbar_init(bar + 8 * i, 1);
     mbar_init(u_begun, 1);
     mbar_init(bar_hit, 1);
+    mbar_init(acc_read, W);
+    mbar_init(recv_read, kCluster * W);
+    mbar_init(bar_end, 1);
     for (int i = 0; i < kSlots; ++i) {
       mbar_init(full + 8 * i, W);
       mbar_init(freed + 8 * i, 1);
@@ -364,6 +392,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   };
   if constexpr (MODE == 3) {
     pdl_wait();
+    deadline = coarse_time() + 3;
     if (warp < W) copy_x();
   }
   if (tid == 0) {
@@ -438,8 +467,10 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
           o[28] = f[n][3];
         }
       }
-      if (tid == 0) mbar_expect(bar_logit, T * 16 * 8);
-      if (tid == NTH + 32) mbar_expect(bar_hit, kCluster * kHitWords * 4);
+      // (nothing is expected while what was expected before is still open)
+      const bool expects = phase_logit == 0 || !broken();
+      if (tid == 0 && expects) mbar_expect(bar_logit, T * 16 * 8);
+      if (tid == NTH + 32 && expects) mbar_expect(bar_hit, kCluster * kHitWords * 4);
       __syncthreads();
       if (!joined) cluster_wait();
       joined = true;
@@ -458,8 +489,9 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
       if (warp < kHitWords) {
         mbar_wait(bar_logit, phase_logit & 1);
         const int t = rank * TR + (tid >> 4), m = tid & 15;
+        const bool whole = !broken();
         float v = 0.0f;
-        if (t < L && m < rrows) {
+        if (t < L && m < rrows && whole) {
           // (in 64 bits: the bias cancels most of the sum of an expert that is just active)
           const double* in = reinterpret_cast<const double*>(smem + lay.off_lrecv) + tid;
           constexpr int s = TR * 16;
@@ -557,15 +589,15 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     } else if (warp < W) {           // the others put the other h buffer back meanwhile
       clear_other(tid - 32 * TR, NTH - 32 * TR);
     }
-    // (twice the limit: a mate whose wait for the logits runs out still says so)
-    mbar_wait(bar_mask, 0, 2);
+    mbar_wait(bar_mask, 0);
+    if (p.hold == 3 && cl == 0 && rank == 1 && lane == 0) ctl[4] = 1;
     const uint32_t flag = lane < T ? tm[words * 32 + lane] : 0u;
     odd_tokens = __ballot_sync(0xffffffffu, flag & 1u);      // with a logit that is not finite
-    // A wait that ran out: out is invalid (this cluster's part is not written). The cluster goes through the
-    // rest with an empty union, so that none of its CTAs is left at a barrier.
+    // A wait for logits that ran out: the four CTAs, all of which have the flags, go through the rest with an
+    // empty union.
     if (__any_sync(0xffffffffu, flag & 2u) && lane == 0) ctl[5] = 1;
     __syncthreads();
-    lost = ctl[5] != 0;                  // (the same for all threads)
+    lost = (ctl[4] | ctl[5]) != 0;                  // (the same for all threads)
     nu = union_of_masks(tm, L, words, ids_sm, ctl);
     if (lost) nu = 0;
   } else {
@@ -589,13 +621,17 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
   const int SD = min(kSlots, lay.off_x / kDSlot), SH = min(kSlots, (lay.off_bar - lay.off_x) / C::kHSlot);
   const uint32_t acc = tmem + 2 * T;
   // (what the two warps below wait for comes behind x: their limits must not run while the call before does)
-  if (MODE != 3 && warp >= W) pdl_wait();
+  if (MODE != 3 && warp >= W) {
+    pdl_wait();
+    deadline = coarse_time() + 3;
+  }
 
   if (warp == W) {
     // ======== the warp that feeds the tensor core ========
     int slot = 0, round = 0;
     for (int ps = 0; ps < npass; ++ps) {
       const int nr = min(rmax, nrows - ps * rmax);
+      if (ps > 0) mbar_wait(acc_read, (ps - 1) & 1);
       for (int kb = 0; kb < nkb; ++kb) {
         mbar_wait(full + 8 * slot, round & 1);
         fence_async();
@@ -614,12 +650,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
           ++round;
         }
       }
-      if (ps + 1 < npass) {
-        cluster_arrive();
-        cluster_wait();
-      } else {
-        tc_commit(u_done);
-      }
+      if (ps + 1 == npass) tc_commit(u_done);
     }
     slot = round = 0;
     int hs = 0, hround = 0;
@@ -645,6 +676,12 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         ++round;
       }
     }
+    if (__any_sync(0xffffffffu, broken())) {       // (nobody may have seen the newest products complete)
+      tc_commit(bar_end);
+      SpinBound limit;
+      while (!mbar_try(bar_end, 0) && !limit.expired(p)) {
+      }
+    }
     __syncwarp();
     cluster_arrive();
   } else if (warp == W + 1) {
@@ -657,19 +694,16 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
                    "r"(ncols * d_e * 2)
                    : "memory");
     __syncwarp();
-    for (int ps = 0; ps + 1 < npass; ++ps) {
-      cluster_arrive();
-      cluster_wait();
-    }
     // (a cluster without rows still copies D: the router's partial sums were there, and no fence for the
     // tensor core has come between them and these copies)
     if (npass > 0)
       mbar_wait(u_done, 0);
     else
       fence_async();
-    int slot = 0, round = 0;
-    for (int s = 0; s < nsw; ++s) {
+    int slot = 0, round = 0, s = 0;
+    for (; s < nsw; ++s) {
       if (s >= SD) mbar_wait(freed_d + 8 * slot, (round - 1) & 1);
+      if (__any_sync(0xffffffffu, broken())) break;
       if (elect_one()) {
         const int n = min(4, nb - 4 * s);
         mbar_expect(full_d + 8 * slot, n * kDBlock);
@@ -688,6 +722,14 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         ++round;
       }
     }
+    if (__any_sync(0xffffffffu, broken())) {       // (nobody may have seen the newest copies land)
+      for (int k = max(0, s - SD); k < s; ++k) {
+        SpinBound limit;
+        while (!mbar_try(full_d + 8 * (k % SD), (k / SD) & 1) && !limit.expired(p)) {
+        }
+      }
+      __syncwarp();
+    }
     cluster_arrive();
   } else {
     // ======== the warps that copy, add and store ========
@@ -704,6 +746,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     };
     auto rest_of_inputs = [&]() {  // MODE 0, 1: what the work before may have written, and the scores of this CTA's tokens
       pdl_wait();
+      deadline = coarse_time() + 3;
       copy_x();
       after_wait();
       if (warp < TR && rank * TR + warp < L)
@@ -730,7 +773,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
           ++iround;
         }
       };
-      if (tid == 0) mbar_expect(bar_up, nr * T * 4);
+      if (tid == 0 && (ps == 0 || !broken())) mbar_expect(bar_up, nr * T * 4);
       if (MODE == 3 && ps == 0) mark_tokens();
       // A stage is handed on when it has landed, `lag` stages (64 to 80 KB) behind the one asked for.
       const int lag = max(1, min(S - 1, kLagBytes / slot_bytes));
@@ -758,14 +801,16 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
           ++round;
         }
       }
+      if (ps > 0) wait_for([&]() { return mbar_try_cluster(recv_read, (ps - 1) & 1); });   // the cluster has read the pass before
       tc_after();
       // partial sums: a lane has a row, a warp 8 tokens; to the CTA that finishes the token
       {
+        const bool sends = !broken();
         const int quad = warp & 3, cg = warp >> 2;
         auto send = [&](uint32_t from, int m, bool ok) {
           uint32_t v[8];
           tc_ld8(v, from + 8 * cg + ((uint32_t)(32 * quad) << 16));
-          if (ok) {
+          if (ok && sends) {
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
               const int tq = 2 * cg + k, to = tq / QR, q = tq % QR;
@@ -785,7 +830,11 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         }
         tc_before();
       }
+      if (ps + 1 < npass) {        // (every lane is past its reads: send ends with a __syncwarp)
+        if (lane == 0) mbar_arrive(acc_read);
+      }
       mbar_wait(bar_up, ps & 1);
+      const bool whole = !broken();
       for (int i0 = 0; i0 < nr * QR; i0 += NTH) {
         const int i = i0 + tid;
         const bool ok = i < nr * QR;
@@ -814,22 +863,21 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         const uint32_t got2 = __shfl_xor_sync(0xffffffffu, o2 ? ta : tb, 2), own2 = o2 ? tb : ta;
         const int t = t0 + 2 * (o1 ? 1 : 0) + (o2 ? 1 : 0);
         const int rb = r & ~3, j = rb - (qe << sh);
-        if (ok && t < L)
+        if (ok && t < L && whole)
           asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(
                            hbuf + ((((size_t)(qe << pshift) + (j >> 6)) * L + t) << 6) + (j & 63)),
                        "r"(o2 ? got2 : own2), "r"(o2 ? own2 : got2)
                        : "memory");
       }
-      if (ps + 1 < npass) {        // the receive buffer is free for the next rows
+      if (ps + 1 < npass) {        // this warp has read the receive buffer
         __syncwarp();
-        cluster_arrive();
-        cluster_wait();
+        if (lane < kCluster) mbar_arrive_cluster(map_rank(recv_read, lane));
       }
     }
     if (MODE == 3 && npass == 0) mark_tokens();
     if (MODE != 3 && npass == 0) rest_of_inputs();
     if (MODE != 3) clear_other(tid, NTH);
-    if (tid == 0) mbar_expect(bar_out, ncols * T * 4);
+    if (tid == 0) mbar_expect(bar_out, ncols * T * 4 + kCluster * 4);
     copy_sync();
 
     // ---- down projection ----
@@ -839,6 +887,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     // is a NaN. Where the scores are given nothing is known about x, and all of h is fetched.)
     constexpr int kHS = NTG == 4 ? 6 : 4;
     const int hj = tid / (4 * T), ht = (tid >> 2) & (T - 1), hp = tid & 3;
+    const bool held = p.hold == 2 || (p.hold == 4 && cl == 0 && rank == 1);
     bool dead = false;
     SpinBound bound;
     int hs = 0, hround = 0;
@@ -860,7 +909,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
           if ((pend >> k) & 1u) ld_relaxed_v8(f[k], h_at + k * h_step);
 #pragma unroll
         for (int k = 0; k < kHS; ++k)
-          if (((pend >> k) & 1u) && !unwritten(f[k]) && p.hold != 2) pend &= ~(1u << k);
+          if (((pend >> k) & 1u) && !unwritten(f[k]) && !held) pend &= ~(1u << k);
       };
       look();
 #pragma unroll
@@ -869,6 +918,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         if (s < nsw) {
           while (!dead && __any_sync(0xffffffffu, (pend >> k) & 1u)) {
             dead = __any_sync(0xffffffffu, bound.expired(p));
+            if (dead) ctl[5] = 1;    // (seen by whoever waits for the products with what is stored below)
             look();
           }
           if (hround > 0) mbar_wait(freed_h + 8 * hs, (hround - 1) & 1);
@@ -886,10 +936,7 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
         }
       }
     }
-    if (dead) {
-      ctl[5] = 1;
-      if (lane == 0) atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
-    }
+    if (dead && lane == 0) atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
     // routing results, spread over clusters: a CTA has its tokens' scores
     if (MODE == 3 && !lost) {
       for (int i = GC - 1 - cl; i < TR; i += GC) {
@@ -919,11 +966,17 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
       }
       tc_before();
     }
+    // whether they are worth anything
+    const uint32_t out_flags = lay.off_hit + kCluster * C::TR / 2 * 4;
+    if (tid < kCluster)
+      st_async_b32(map_rank(sbase + out_flags + rank * 4, tid),
+                   *reinterpret_cast<const volatile uint32_t*>(ctl + 5) | (broken() ? 1u : 0u), map_rank(bar_out, tid));
     __syncwarp();
     cluster_arrive();
     mbar_wait(bar_out, 0);
     copy_sync();
-    if (ctl[5] == 0 && has_out) {
+    const uint4 bad = lds128(sbase + out_flags);
+    if (!broken() && (bad.x | bad.y | bad.z | bad.w) == 0 && has_out) {
       const int t = tid >> 6;
       const float* r = reinterpret_cast<const float*>(smem + lay.off_drecv) + ((t >> 2) * kDRows + om) * 4 + (t & 3);
       constexpr int s = QR * kDRows * 4;
@@ -958,6 +1011,13 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(C::kTmem));
   }
   cluster_wait();                  // nobody sends to this CTA any more
+  if (broken()) {
+    if (tid == 0) atomicOr(p.status, BLOCKFFN_DEV_WAIT_EXPIRED);
+    // (what it sent last may be on its way yet, for 0.2 us, and no wait has covered it)
+    const unsigned long long t0 = clock_ns();
+    while (clock_ns() - t0 < 100000ull) {
+    }
+  }
 }
 
 // ---- host side -------------------------------------------------------------------------------
@@ -1119,7 +1179,9 @@ cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, co
   const int groups = (c->cfg.E + 15) / 16;
   p.reps = pl.clusters >= groups ? pl.clusters / groups : 1;
   p.hold = !(c->cfg.flags & BLOCKFFN_CFG_TEST_EXPIRE_WAIT) ? 0 : scores || (c->cfg.flags & BLOCKFFN_CFG_NO_SPLIT) ? 2 : 1;
+  if (p.hold && (c->cfg.flags & BLOCKFFN_CFG_NO_CHAINING)) p.hold += 2;
   p.wait_ns = 1000000000ull;      // one second
+  p.time_shift = p.hold ? 22 : 31;
   p.status = c->status;
   if (pub) p.pub = *pub;
   cudaLaunchConfig_t lc{};

@@ -194,3 +194,45 @@ def test_a_call_behind_one_that_gives_up(L):
         call(out, 0)
         assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
         assert bool((held == 7.0).all()) and torch.equal(out, want)
+
+
+@pytest.mark.parametrize("kind", ["masks", "h, router on", "h, scores", "h, list"])
+@pytest.mark.parametrize("L", [12, 32])
+def test_one_cta_that_gives_up(L, kind):
+    """One CTA of the first cluster runs out of time alone, rows of U being in several passes. With the union not
+    known to it, the intermediate stays incomplete and nobody writes out; with h missing, its cluster's columns
+    are not written and the others are as always. All come to their end, and the next calls are right."""
+    d, E, d_e = 2048, 128, 128
+    layer, dw = B.Layer(d, E, d_e, L_max=32), make(d, E, d_e, 4, 9.0)
+    cfg = B.Config.from_address(layer.h.value)
+    assert (cfg.d, cfg.E, cfg.d_e, cfg.L_max, cfg.flags) == (d, E, d_e, 32, 0)
+    x = torch.randn(L, d, device="cuda").bfloat16()
+    scores = torch.rand(L, E, device="cuda") + 0.1
+    ids, n = torch.arange(E, dtype=torch.int32, device="cuda"), torch.tensor([E], dtype=torch.int32, device="cuda")
+    flags = B.CFG_TEST_EXPIRE_WAIT | B.CFG_NO_CHAINING | (B.CFG_NO_SPLIT if kind == "h, router on" else 0)
+
+    def call(o):
+        if kind in ("masks", "h, router on"):
+            B.blockffn_layer_forward(layer.h, dw.struct, x, L, o)
+        elif kind == "h, scores":
+            B.blockffn_layer_forward_scores(layer.h, dw.struct, x, scores, L, o)
+        else:
+            B.blockffn_expert_ffn(layer.h, dw.struct, x, scores, L, ids, n, o)
+    want, out = (torch.full((L, d), 7.0, device="cuda") for _ in range(2))
+    call(want)
+    assert layer.last_status() == 0 and not bool((want == 7.0).all(0).any())
+    for _ in range(3):
+        out.fill_(7.0)
+        cfg.flags = flags
+        call(out)
+        cfg.flags = 0
+        assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+        untouched = (out == 7.0).all(0)
+        if kind == "masks":
+            assert bool(untouched.all())
+        else:
+            c = int(untouched.sum())
+            assert 1 < c <= 64 and bool(untouched[:c].all()) and torch.equal(out[:, c:], want[:, c:])
+        out.fill_(7.0)
+        call(out)
+        assert torch.equal(out, want) and layer.last_status() == 0
