@@ -145,6 +145,13 @@ cudaError_t launch_expert_chain(blockffn_ctx* c, const blockffn_weights* w, cons
                                 float* out, void* x_next, int call_flags, const RoutingOut* pub,
                                 cudaStream_t st);
 
+// Elements of U of the experts that the caller expects in a chunk's union (by default 30 % of all).
+inline long long expected_union_elements(const blockffn_ctx* c) {
+  int u = (c->cfg.flags >> 17) & 0x7ff;
+  if (u == 0) u = (3 * c->cfg.E + 5) / 10;
+  return (long long)u * c->cfg.d_e * c->cfg.d;
+}
+
 // The same for longer chunks, on clusters of four CTAs (expert_cluster.cu), with the router inside
 // (scores == NULL) or scores and maybe the union list given.
 bool expert_cluster_supported(const blockffn_ctx* c, int L, bool router);

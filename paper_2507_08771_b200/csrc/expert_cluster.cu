@@ -1061,9 +1061,7 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
 //     32 tokens 24.2 / 16.9
 //   scores given, 9 to 16: from 6 M. d = 2048, E = 64 (5 M) 8.8 / 8.7; E = 128 (10 M), 16 tokens 19.5 / 15.6
 ClusterPlan cluster_plan(const blockffn_ctx* c, int L, bool router) {
-  int u_exp = (c->cfg.flags >> 17) & 0x7ff;
-  if (u_exp == 0) u_exp = (3 * c->cfg.E + 5) / 10;
-  const long long u = (long long)u_exp * c->cfg.d_e * c->cfg.d;
+  const long long u = expected_union_elements(c);
   if (L > 16 && L <= 32 && (router || u >= 4000000)) return cluster_plan_of<4>(c->cfg, L, c->clusters);
   if (L > 8 && L <= 16 && u >= 6000000) return cluster_plan_of<2>(c->cfg, L, c->clusters);
   return ClusterPlan{};

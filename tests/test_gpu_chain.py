@@ -161,6 +161,37 @@ def chain(layer, dws, lengths, h, x, flags, each=lambda i: None):
         each(i)
 
 
+@pytest.mark.parametrize("d,E,d_e", [(64, 40, 64), (128, 64, 64), (192, 128, 128), (192, 24, 256)])
+def test_long_chunks_of_narrow_layers(d, E, d_e):
+    """17 to 32 tokens at widths too small for the clusters, and the same from a handle that expects so few
+    experts that the throughput kernel takes them: one by one, one behind the other, and with a wait that runs out."""
+    # (At -0.5 a third of the experts is active, and the RMS of a token's logits is 0.1 or more: their error, up to
+    # 1e-6, is then within 1e-5 of a score. At -1.6 some tokens have one active logit of a few thousandths, and
+    # 1e-6 of it is 1e-4 of its score: 5e-5 seen, with the 1e-5 of check missed.)
+    dws = [make(d, E, d_e, s, b) for s, b in enumerate((-0.5, 0.3, 9.0, -9.0))]
+    g = torch.Generator(device="cuda").manual_seed(d + E)
+    for cfg in (0, 1 << 17):                      # (bits 17 on: experts expected in the union)
+        layer = B.Layer(d, E, d_e, L_max=32, flags=cfg)
+        for L in (17, 24, 32):
+            x = torch.randn(L, d, device="cuda", generator=g).bfloat16()
+            want = []
+            for dw in dws:
+                check(layer, dw, x, B.CALL_INDEPENDENT)
+                want.append(layer.forward(dw, x, call_flags=B.CALL_INDEPENDENT).out.clone())
+            outs = [torch.empty(L, d, device="cuda") for _ in range(12)]
+            torch.cuda.synchronize()
+            for i, o in enumerate(outs):
+                B.blockffn_layer_forward(layer.h, dws[i % 4].struct, x, L, o, call_flags=B.CALL_INDEPENDENT)
+            assert all(torch.equal(o, want[i % 4]) for i, o in enumerate(outs))
+        assert layer.last_status() == 0
+    held = B.Layer(d, E, d_e, L_max=32, flags=B.CFG_TEST_EXPIRE_WAIT)
+    for _ in range(2):
+        out = torch.full((24, d), 7.0, device="cuda")
+        held.forward(dws[0], torch.randn(24, d, device="cuda").bfloat16(), out=out)
+        assert held.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+        assert bool((out == 7.0).all())
+
+
 @pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
 @pytest.mark.parametrize("lengths", [[1], [8], [13], [16], [32], [1, 32, 8, 17, 9, 24, 3, 16]], ids=str)
 @pytest.mark.parametrize("d,E", [(1024, 40), (2048, 64)])
