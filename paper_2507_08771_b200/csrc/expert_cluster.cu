@@ -1049,21 +1049,32 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
   return pl;
 }
 // Where a call comes here. The hops through distributed shared memory cost a few microseconds that the smaller
-// broadcast and the one pass over the weights have to save, so the line lies at the number of elements of the
-// expected union's U. us per layer of a captured stack, kernel of before / this one (M elements):
-//   router on, 17 to 32 tokens: always. 32 tokens, d = 512, E = 32, d_e = 64 (0.3 M) 11.5 / 11.1; 17 tokens,
-//     d = 1536, E = 48, d_e = 128 (2.8 M) 14.4 / 13.5; 32 tokens, d = 2048, E = 128, d_e = 128 (10 M) 24.8 / 18.3
-//   router on, 9 to 16: from 6 M. 13 tokens, d = 1792, E = 56, d_e = 128 (3.9 M) 11.9 / 12.6; d = 2048, E = 64
-//     (5 M) 12 tokens 13.2 / 13.4, 16 tokens 13.7 / 13.5; E = 96 (7.6 M), 10 tokens 18.4 / 15.7; E = 128 (10 M),
-//     16 tokens 22.2 / 18.1
+// broadcast and the one pass over the weights have to save, so the lines lie at the number of elements of the
+// expected union's U (the hint of the configuration, or 30 % of the experts: the union itself is known on the device
+// only, and a call whose union is another one takes the kernel of the expected one). us per layer of a captured
+// stack, kernel of expert_chain.cu, or with scores given expert_wide.cuh / this one (M elements):
+//   router on, 17 to 32 tokens: below d = 1024 always, above from 24 M elements times tokens. d = 512, E = 16,
+//     d_e = 64 (0.2 M), 17 tokens 11.6 / 11.3; d = 1024, E = 24, d_e = 64 (0.5 M), 24 tokens 11.6 / 12.0; d = 2048, E = 16,
+//     d_e = 64 (0.7 M), 17 tokens 12.8 / 13.4, 32 tokens 13.8 / 13.7; E = 24, d_e = 128 (1.8 M), 17 tokens 13.5 / 13.8,
+//     32 tokens 14.4 / 14.1; d = 1536, E = 48, d_e = 128 (2.8 M), 17 tokens 14.4 / 13.5; d = 2048, E = 128, d_e = 128
+//     (10 M), 32 tokens 24.8 / 18.5
+//   router on, 9 to 16: from 6 M, up to d = 1024 from 9 M. 13 tokens, d = 1792, E = 56, d_e = 128 (3.9 M) 11.9 / 12.6;
+//     d = 2048, E = 64 (5 M) 12 tokens 13.2 / 13.4, 16 tokens 13.7 / 13.5; d = 1536, E = 52, d_e = 256 (6.3 M), 9 tokens
+//     18.4 / 15.4; d = 2048, E = 128 (10 M), 16 tokens 22.2 / 18.5; d = 1024, d_e = 256, E = 80 (6.3 M), 9 tokens 17.2 / 17.9,
+//     E = 100 (7.9 M), 10 tokens 18.9 / 19.4, E = 128 (10 M), 12 tokens 23.1 / 22.9
 //   scores given, 17 to 32: from 4 M. d = 1536, E = 48 (2.9 M), 18 tokens 11.3 / 11.7; d = 2048, E = 100,
 //     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 64, d_e = 128 (5 M), 24 tokens 15.7 / 13.2; E = 128 (10 M),
 //     32 tokens 24.2 / 16.9
 //   scores given, 9 to 16: from 6 M. d = 2048, E = 64 (5 M) 8.8 / 8.7; E = 128 (10 M), 16 tokens 19.5 / 15.6
 ClusterPlan cluster_plan(const blockffn_ctx* c, int L, bool router) {
   const long long u = expected_union_elements(c);
-  if (L > 16 && L <= 32 && (router || u >= 4000000)) return cluster_plan_of<4>(c->cfg, L, c->clusters);
-  if (L > 8 && L <= 16 && u >= 6000000) return cluster_plan_of<2>(c->cfg, L, c->clusters);
+  const int d = c->cfg.d;
+  if (L > 16 && L <= 32) {
+    if (!router && u < 4000000) return ClusterPlan{};
+    if (router && d >= 1024 && u * L < 24000000 && expert_chain_supported(c, L)) return ClusterPlan{};
+    return cluster_plan_of<4>(c->cfg, L, c->clusters);
+  }
+  if (L > 8 && L <= 16 && u >= (router && d <= 1024 ? 9000000 : 6000000)) return cluster_plan_of<2>(c->cfg, L, c->clusters);
   return ClusterPlan{};
 }
 

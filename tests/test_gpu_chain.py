@@ -161,9 +161,9 @@ def chain(layer, dws, lengths, h, x, flags, each=lambda i: None):
         each(i)
 
 
-@pytest.mark.parametrize("d,E,d_e", [(64, 40, 64), (128, 64, 64), (192, 128, 128), (192, 24, 256)])
-def test_long_chunks_of_narrow_layers(d, E, d_e):
-    """17 to 32 tokens at widths too small for the clusters, and the same from a handle that expects so few
+@pytest.mark.parametrize("d,E,d_e", [(64, 40, 64), (128, 64, 64), (192, 128, 128), (192, 24, 256), (1984, 16, 64), (1024, 31, 64)])
+def test_long_chunks_off_the_clusters(d, E, d_e):
+    """17 to 32 tokens at widths or expected unions too small for the clusters, and the same from a handle that expects so few
     experts that the throughput kernel takes them: one by one, one behind the other, and with a wait that runs out."""
     # (At -0.5 a third of the experts is active, and the RMS of a token's logits is 0.1 or more: their error, up to
     # 1e-6, is then within 1e-5 of a score. At -1.6 some tokens have one active logit of a few thousandths, and
