@@ -1,11 +1,12 @@
-"""Router-on layer calls of 17 to 32 tokens (and of 9 to 16 with a large union) behind one another: one
-kernel on clusters of four CTAs. Edges of its K quarters, row tiles and expert groups; references and
-tolerances as in test_gpu_chain."""
+"""Dependent calls of 17 to 32 tokens, and of 9 to 16 with a large union, as one kernel on clusters of four CTAs:
+router on, scores given, a list given. Edges of its K quarters, row tiles and expert groups, calls one behind
+the other, and calls that give up; references and tolerances as in test_gpu_chain. (That a shape takes this kernel
+shows in test_one_cta_that_gives_up: in the others, all CTAs give up or none.)"""
 import pytest
 import torch
 
 from paper_2507_08771_b200 import binding as B
-from test_gpu_chain import check, make, reference
+from test_gpu_chain import chain, check, layers, make, reference
 
 pytestmark = pytest.mark.gpu
 
@@ -104,6 +105,47 @@ def test_scores_given(d, E, d_e, L, flags, listed):
             assert bool(out[L - 1].isnan().all())
 
 
+@pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
+@pytest.mark.parametrize("lengths", [[12], [16], [32], [16, 32, 9, 17, 8, 13]], ids=str)
+def test_router_on_one_behind_the_other(lengths, flags):
+    """As test_calls_one_behind_the_other of test_gpu_chain, with unions large enough for chunks of 9 to 16
+    tokens, whose CTAs are on the SMs two calls at a time."""
+    d, E, d_e = 2048, 128, 128
+    dws, layer = layers(E, d, d_e), B.Layer(d, E, d_e, L_max=32)
+    lengths = (lengths * 20)[:20]
+    start = torch.randn(32, d, device="cuda")
+    h, x = start.clone(), torch.zeros(2, 32, d, dtype=torch.bfloat16, device="cuda")
+
+    def run(each=lambda i: None):
+        h.copy_(start)
+        x.copy_(start.expand(2, 32, d))
+        chain(layer, dws, lengths, h, x, flags, each)
+        return h.clone(), x.clone()
+    seen = {"h": start.double(), "x": start.bfloat16()}
+
+    def compare(i):
+        L = lengths[i]
+        torch.cuda.synchronize()
+        _, ref = reference(dws[i % len(dws)].tensors, seen["x"][:L])
+        rms = max(ref.square().mean().sqrt().item(), 1e-6)
+        assert (h[:L].double() - seen["h"][:L] - ref).abs().max().item() <= 2e-2 * rms + 1e-5
+        seen["h"], seen["x"] = h.double(), x[(i + 1) % 2].clone()
+    want = run(compare)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        h.copy_(start)
+        x.copy_(start.expand(2, 32, d))
+        chain(layer, dws, lengths, h, x, flags)
+    for _ in range(3):
+        graph.replay()
+        got = run()
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(h, want[0]) and torch.equal(x, want[1]) and layer.last_status() == 0
+
+
 @pytest.mark.parametrize("listed", [False, True])
 @pytest.mark.parametrize("d,E,d_e,L", [(2048, 128, 128, 12), (2048, 64, 256, 16), (2048, 64, 128, 20), (2048, 128, 128, 32)])
 def test_scores_given_one_behind_the_other(d, E, d_e, L, listed):
@@ -194,6 +236,30 @@ def test_a_call_behind_one_that_gives_up(L):
         call(out, 0)
         assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
         assert bool((held == 7.0).all()) and torch.equal(out, want)
+
+
+@pytest.mark.parametrize("kind", ["logits", "h, router on", "scores", "list"])
+@pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
+@pytest.mark.parametrize("L", [12, 32])
+def test_all_ctas_that_give_up(L, flags, kind):
+    """The bounded waits, for logits and for the intermediate, in every form of the kernel: out stays as it was."""
+    d, E, d_e = 2048, 128, 128
+    held = B.Layer(d, E, d_e, L_max=L, flags=B.CFG_TEST_EXPIRE_WAIT | (B.CFG_NO_SPLIT if kind == "h, router on" else 0))
+    dw, x = make(d, E, d_e, 2, -0.5), torch.randn(L, d, device="cuda").bfloat16()
+    scores = torch.rand(L, E, device="cuda") * (torch.arange(E, device="cuda") % 3 == 0)
+    ids = torch.arange(E, dtype=torch.int32, device="cuda") * 3 % E
+    n = torch.tensor([E // 3], dtype=torch.int32, device="cuda")
+    out = torch.full((L, d), 7.0, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(3):
+        if kind in ("logits", "h, router on"):
+            B.blockffn_layer_forward(held.h, dw.struct, x, L, out, call_flags=flags)
+        elif kind == "scores":
+            B.blockffn_layer_forward_scores(held.h, dw.struct, x, scores, L, out, call_flags=flags)
+        else:
+            B.blockffn_expert_ffn(held.h, dw.struct, x, scores, L, ids, n, out, call_flags=flags)
+        assert held.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+        assert bool((out == 7.0).all())
 
 
 @pytest.mark.parametrize("kind", ["masks", "h, router on", "h, scores", "h, list"])

@@ -39,11 +39,11 @@ def test_calls_with_and_without_a_promise(L):
 
 @pytest.mark.parametrize("L", [16, 32])
 @pytest.mark.parametrize("graph", [False, True])
-def test_calls_without_a_promise_beside_other_streams(L, graph):
+@pytest.mark.parametrize("d,E,d_e,n", [(1024, 32, 64, 40), (2048, 128, 128, 20)])     # the one-kernel form; clusters
+def test_calls_without_a_promise_beside_other_streams(d, E, d_e, n, L, graph):
     """Two handles' calls on streams of different priorities beside a stream of large products: every
     call gets its places on the SMs as a whole, none gives up waiting, and the results are those of
     the same calls alone."""
-    d, E, d_e, n = 1024, 32, 64, 40
     dws = [make(d, E, d_e, s, 0.0) for s in range(2)]
     layers = [B.Layer(d, E, d_e, L_max=L) for _ in range(2)]
     x = [torch.randn(L, d, device="cuda").bfloat16() for _ in range(2)]
@@ -86,8 +86,8 @@ def test_calls_without_a_promise_beside_other_streams(L, graph):
 
 
 @pytest.mark.parametrize("d,E,L,want", [
-    (2048, 544, 32, 1), (1024, 992, 32, 1), (2048, 712, 24, 1), (2048, 952, 17, 1),   # no pools of the chain kernel
-    (512, 1024, 16, 1), (512, 1024, 32, 1),                                           # the chain kernel
+    (2048, 544, 32, 1), (1024, 992, 32, 1), (2048, 712, 24, 1), (2048, 952, 17, 1),   # (too many experts for the pools of the chain kernel)
+    (512, 1024, 16, 1), (512, 1024, 32, 1),                                           # up to 16 tokens the chain kernel, above clusters
 ])
 @pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
 def test_dependent_router_on_calls_of_many_experts(d, E, L, want, flags):

@@ -190,8 +190,8 @@ def test_expert_ffn_under_call_promises(kind, d, E, d_e, L, p):
     """The expert stage under the two per-call promises. With x promised stable the one-kernel form
     runs a call on about a third of the SMs (up to three column tiles of out and several stages per
     CTA); with only the weights promised stable it owns the device (up to 8 tokens: the up/down
-    pair; longer chunks: the one-kernel form, which then waits for its predecessor before it reads
-    x). Shapes cover one to three column tiles, one and several stages, unions from a few experts
+    pair; longer chunks: the one-kernel form, or with a large expected union the kernel on clusters, which
+    then wait for their predecessor before they read x). Shapes cover one to three column tiles, one and several stages, unions from a few experts
     to all of them, and chunks of 9 to 32 tokens (two token groups per weight fragment; from 17
     tokens on two teams of them in one CTA)."""
     seed = 3000 + d + E + L
@@ -579,8 +579,8 @@ def check_layer_router_on(layer, dw, w, x, L, bias=None, want_out=False, call_fl
 @pytest.mark.parametrize("L", [9, 16, 17, 32])
 def test_router_on_long_chunks(L, flag):
     """blockffn_layer_forward on chunks of more than 8 tokens: the router runs inside the
-    long-chunk kernel (8 tokens per pass), with and without the x-stable promise; several calls
-    in a row on one handle."""
+    long-chunk kernel (8 tokens per pass) with the x-stable promise, inside the dependent-chain kernel or the one
+    on clusters without; several calls in a row on one handle."""
     sh, seed = I.SHAPES[3], I.config_seed(3)
     w = I.make_layer(sh, seed, bias_shift=I.ROUTER_BIAS_SHIFT)
     layer = B.Layer(sh.d, sh.E, sh.d_e, L_max=32)
@@ -801,7 +801,7 @@ def test_bench_launch_configuration_stack(L):
     """Config 4 as the benchmark runs it: residual accumulate, bf16 hand-over between layers,
     CALL_INDEPENDENT on every layer call, one graph; compared with the oracle's stack. Chunks of
     more than 8 tokens take the one-kernel form in its dependent-chain mode (it waits for the
-    layer before, then reads x), shorter ones the up/down pair."""
+    layer before, then reads x), those of 32 tokens clusters, shorter ones the up/down pair."""
     sh, seed = I.SHAPES[4], I.config_seed(4)
     n_layers, L = (5, sh.L) if L is None else (4, L)
     layer = B.Layer(sh.d, sh.E, sh.d_e, L_max=L)
