@@ -41,7 +41,7 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
   const bool x_stable = logits ? logits_final : (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
   const bool dep_long = !x_stable && !logits && L > 8;
   const bool dep_inside = !x_stable && logits && logits->a0 == nullptr;   // router inside the kernel
-  if (dep_long && expert_cluster_supported(c, L, false)) {
+  if (dep_long && expert_cluster_supported(c, L, union_ids ? 1 : 0)) {
     const cudaError_t e = launch_expert_cluster(c, w, x, scores, L, union_ids, n_union, out, x_next,
                                                 call_flags, pub, st);
     if (e != cudaErrorCooperativeLaunchTooLarge) return e;
@@ -312,7 +312,7 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     // calls never writes what their kernels still read.
     const bool x_stable_call = (call_flags & BLOCKFFN_CALL_INDEPENDENT_X) != 0;
     const RoutingOut pub_in{h->union_mask, h->union_ids, h->n_union, stats, h->scores, h->tok_mask};
-    if (!x_stable_call && expert_cluster_supported(h, L, true)) {
+    if (!x_stable_call && expert_cluster_supported(h, L, 3)) {
       // x from the call before: one kernel made for that chain, router included
       h->last_layer_waited_first = false;
       return launch_expert_cluster(h, w, x, nullptr, L, nullptr, nullptr, out, x_next, call_flags, &pub_in, st) == cudaSuccess

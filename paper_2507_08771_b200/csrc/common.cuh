@@ -154,7 +154,8 @@ inline long long expected_union_elements(const blockffn_ctx* c) {
 
 // The same for longer chunks, on clusters of four CTAs (expert_cluster.cu), with the router inside
 // (scores == NULL) or scores and maybe the union list given.
-bool expert_cluster_supported(const blockffn_ctx* c, int L, bool router);
+// mode: 0 scores given, 1 scores and list given, 3 router on.
+bool expert_cluster_supported(const blockffn_ctx* c, int L, int mode);
 cudaError_t expert_cluster_setup(blockffn_ctx* c);
 cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x,
                                   const float* scores, int L, const int32_t* union_ids,

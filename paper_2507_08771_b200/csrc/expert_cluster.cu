@@ -1063,18 +1063,29 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
 //     18.4 / 15.4; d = 2048, E = 128 (10 M), 16 tokens 22.2 / 18.5; d = 1024, d_e = 256, E = 80 (6.3 M), 9 tokens 17.2 / 17.9,
 //     E = 100 (7.9 M), 10 tokens 18.9 / 19.4, E = 128 (10 M), 12 tokens 23.1 / 22.9
 //   scores given, 17 to 32: from 4 M. d = 1536, E = 48 (2.9 M), 18 tokens 11.3 / 11.7; d = 2048, E = 100,
-//     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 64, d_e = 128 (5 M), 24 tokens 15.7 / 13.2; E = 128 (10 M),
-//     32 tokens 24.2 / 16.9
-//   scores given, 9 to 16: from 6 M. d = 2048, E = 64 (5 M) 8.8 / 8.7; E = 128 (10 M), 16 tokens 19.5 / 15.6
-ClusterPlan cluster_plan(const blockffn_ctx* c, int L, bool router) {
+//     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 54, d_e = 128 (4.2 M), 17 tokens 13.1 / 12.4; E = 64 (5 M), 24 tokens
+//     15.7 / 13.2; E = 128 (10 M), 32 tokens 24.2 / 16.9. A list given: from 4.5 M (it is known sooner than a union that
+//     has to be derived, which the other kernel is the better for). d = 2048, 17 tokens, E = 104, d_e = 64 (4.1 M)
+//     10.6 / 11.6; E = 64, d_e = 128 (5 M), 24 tokens, nothing promised 14.1 / 12.6
+//   scores given, 9 to 16: from 6 M, and from 9.3 G elements times d: the 64 columns of D that are copied at a time are a
+//     cluster's own at d = 2048 and twice those at d = 1024. d = 2048, E = 64 (5 M) 8.8 / 8.7; E = 80 (6.3 M), 9 tokens
+//     12.5 / 11.6; E = 128 (10 M), 16 tokens 20.1 / 16.1; d = 1536, E = 52, d_e = 256 (6.3 M), 9 tokens 12.2 / 12.1;
+//     d = 1024, d_e = 256, 9 tokens, E = 80 (6.3 M) 12.9 / 15.4, E = 128 (10 M) 21.5 / 21.0; d = 512, E = 128, d_e = 512
+//     (10 M), 9 tokens 27.2 / 32.5. A list given: from 12 G. d = 1536, E = 110, d_e = 128 (6.5 M), 9 tokens 9.3 / 10.8,
+//     16 tokens 10.4 / 10.9; d = 2048, E = 80 (6.3 M) 9.3 / 9.7 and 10.3 / 10.0, E = 128 (10 M) 15.5 / 14.3 and 16.5 / 14.6
+ClusterPlan cluster_plan(const blockffn_ctx* c, int L, int mode) {
   const long long u = expected_union_elements(c);
   const int d = c->cfg.d;
   if (L > 16 && L <= 32) {
-    if (!router && u < 4000000) return ClusterPlan{};
-    if (router && d >= 1024 && u * L < 24000000 && expert_chain_supported(c, L)) return ClusterPlan{};
+    if (mode == 3 ? d >= 1024 && u * L < 24000000 && expert_chain_supported(c, L) : u < (mode == 1 ? 4500000 : 4000000))
+      return ClusterPlan{};
     return cluster_plan_of<4>(c->cfg, L, c->clusters);
   }
-  if (L > 8 && L <= 16 && u >= (router && d <= 1024 ? 9000000 : 6000000)) return cluster_plan_of<2>(c->cfg, L, c->clusters);
+  if (L > 8 && L <= 16) {
+    if (mode == 3 ? u < (d <= 1024 ? 9000000 : 6000000) : u < 6000000 || u * d < (mode == 1 ? 12000000000 : 9300000000))
+      return ClusterPlan{};
+    return cluster_plan_of<2>(c->cfg, L, c->clusters);
+  }
   return ClusterPlan{};
 }
 
@@ -1117,9 +1128,9 @@ cudaError_t cluster_attr() {
 
 }  // namespace
 
-bool expert_cluster_supported(const blockffn_ctx* c, int L, bool router) {
+bool expert_cluster_supported(const blockffn_ctx* c, int L, int mode) {
   if (c->chain_ws == nullptr || (c->cfg.flags & BLOCKFFN_CFG_TWO_KERNELS)) return false;
-  return cluster_plan(c, L, router).ok;
+  return cluster_plan(c, L, mode).ok;
 }
 
 // How many clusters fit the device at one CTA per SM (0: none do, or no chunk length takes them).
@@ -1149,7 +1160,8 @@ cudaError_t expert_cluster_setup(blockffn_ctx* c) {
 cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, const void* x, const float* scores,
                                   int L, const int32_t* union_ids, const int32_t* n_union, float* out,
                                   void* x_next, int call_flags, const RoutingOut* pub, cudaStream_t st) {
-  const ClusterPlan pl = cluster_plan(c, L, scores == nullptr);
+  const int mode = !scores ? 3 : union_ids ? 1 : 0;
+  const ClusterPlan pl = cluster_plan(c, L, mode);
   if (!pl.ok || !c->chain_ws) return cudaErrorNotSupported;
   const ChainWorkspace ws = chain_workspace(c);
   ClusterParams p{};
@@ -1214,7 +1226,6 @@ cudaError_t launch_expert_cluster(blockffn_ctx* c, const blockffn_weights* w, co
                            steps, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  const int mode = !scores ? 3 : union_ids ? 1 : 0;
   const cudaError_t e = pl.ntg == 4 ? mode == 3   ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<4, 3>, p, map)
                                       : mode == 1 ? cudaLaunchKernelEx(&lc, expert_cluster_kernel<4, 1>, p, map)
                                                   : cudaLaunchKernelEx(&lc, expert_cluster_kernel<4, 0>, p, map)
