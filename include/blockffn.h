@@ -31,7 +31,8 @@
  *     once, at most one per SM: blockffn_layer_forward, and scores-in or list calls with one of
  *     the two promises below (the INDEPENDENT flags). Such calls of two handles on two streams
  *     are fine while other work lets go of the SMs in time; a call that cannot get its SMs
- *     within a second gives up (BLOCKFFN_DEV_WAIT_EXPIRED). A program that shares the GPU with
+ *     within a second gives up (BLOCKFFN_DEV_WAIT_EXPIRED). (Longer dependent chunks run on clusters
+ *     of four CTAs: those need their four SMs from one group of SMs, all four at a time.) A program that shares the GPU with
  *     kernels that hold SMs for that long, or that runs several handles' calls at the same time
  *     on streams of different priorities, sets BLOCKFFN_CFG_TWO_KERNELS: no kernel then waits
  *     for another CTA. Scores-in and list calls without a promise do not have that condition: of

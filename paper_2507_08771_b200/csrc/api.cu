@@ -328,10 +328,10 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
     if ((x_stable_call || L > 8) && expert_lean_supported(h, L, true, x_stable_call, true)) {
       // x stable: the router runs inside the one-kernel form (its CTAs share the experts' logits
       // out between them and exchange them through L2), so the call is one launch that overlaps
-      // its neighbours like a scores-in call. A dependent call comes here where the score matrix
-      // leaves the chain kernel no room for its pools (17 to 32 tokens of about a thousand experts):
-      // one launch on the whole device. d_e = 64: 117 us per layer at d = 1024, E = 992, 32 tokens
-      // against 243 for the router and the pair; 112 against 171 at d = 2048, E = 800, 24 tokens.
+      // its neighbours like a scores-in call. A dependent call of more than 8 tokens comes here where
+      // neither kernel above takes it: 17 to 32 tokens with hardly anything to fetch (expert_chain_supported
+      // has the figures), or a score matrix too large for the chain kernel's pools where the clusters do not
+      // take the shape. One launch on the whole device.
       const RouterLogits lg_in{nullptr, router_gain(h, w), h->cfg.rms_eps};
       h->last_layer_waited_first = false;
       return launch_tensor_core(h, w, x, h->scores, L, nullptr, nullptr, out, x_next, flags, &pub_in,

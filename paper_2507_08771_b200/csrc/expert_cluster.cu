@@ -1,6 +1,7 @@
 // A layer call of 9 to 32 tokens in a dependent chain (x is what the call before left) as one kernel on
 // clusters of four CTAs: router (Eq. 3), or scores and maybe the union list given, Union(x) (Sec. 3.3), up and
-// down projection (Eq. 1, Eq. 2); chunks of up to 16 tokens where the union is large (cluster_plan). The steps and the two exchanges over the whole device are those of
+// down projection (Eq. 1, Eq. 2). Which calls come here: cluster_plan, below. The steps and the two exchanges
+// over the whole device are those of
 // expert_chain.cu (which see); this file is about what 32 tokens cost there: every CTA took in all
 // of x and of h, 128 + 344 KB, next to 290 KB of weights, and 16 warps fed mma.sync from registers,
 // so that a layer was bound by issue slots (22.6 K of its 46 K cycles per scheduler), by L2 -> SM
@@ -801,7 +802,8 @@ __global__ void __launch_bounds__(Dims<NTG>::NTH + 64, NTG == 4 ? 1 : 2)
           ++round;
         }
       }
-      if (ps > 0) wait_for([&]() { return mbar_try_cluster(recv_read, (ps - 1) & 1); });   // the cluster has read the pass before
+      // (the cluster has read the pass before)
+      if (ps > 0) wait_for([&]() { return mbar_try_cluster(recv_read, (ps - 1) & 1); });
       tc_after();
       // partial sums: a lane has a row, a warp 8 tokens; to the CTA that finishes the token
       {

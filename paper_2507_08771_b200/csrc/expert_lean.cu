@@ -1,6 +1,6 @@
 // Expert stage (Eq. 1, Eq. 2 restricted to Union(x), Sec. 3.3) as one kernel per call, for
 // calls whose inputs are all stable (x included), so that several calls are in flight per SM,
-// and for all chunks of more than 8 tokens with scores given.
+// and for dependent chunks of more than 8 tokens with scores given (large unions: expert_cluster.cu).
 // expert_lean_kernel takes chunks of up to 8 tokens, expert_wide_kernel (expert_wide.cuh) chunks
 // of 9 to 32.
 //

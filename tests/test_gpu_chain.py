@@ -170,7 +170,7 @@ def test_long_chunks_off_the_clusters(d, E, d_e):
     # 1e-6 of it is 1e-4 of its score: 5e-5 seen, with the 1e-5 of check missed.)
     dws = [make(d, E, d_e, s, b) for s, b in enumerate((-0.5, 0.3, 9.0, -9.0))]
     g = torch.Generator(device="cuda").manual_seed(d + E)
-    for cfg in (0, 1 << 17):                      # (bits 17 on: experts expected in the union)
+    for cfg in (0, B.cfg_expected_union(1)):
         layer = B.Layer(d, E, d_e, L_max=32, flags=cfg)
         for L in (17, 24, 32):
             x = torch.randn(L, d, device="cuda", generator=g).bfloat16()

@@ -86,8 +86,9 @@ def test_calls_without_a_promise_beside_other_streams(d, E, d_e, n, L, graph):
 
 
 @pytest.mark.parametrize("d,E,L,want", [
-    (2048, 544, 32, 1), (1024, 992, 32, 1), (2048, 712, 24, 1), (2048, 952, 17, 1),   # (too many experts for the pools of the chain kernel)
-    (512, 1024, 16, 1), (512, 1024, 32, 1),                                           # up to 16 tokens the chain kernel, above clusters
+    # clusters (too many experts for the pools of the chain kernel)
+    (2048, 544, 32, 1), (1024, 992, 32, 1), (2048, 712, 24, 1), (2048, 952, 17, 1),
+    (512, 1024, 16, 1), (512, 1024, 32, 1),          # the chain kernel, clusters
 ])
 @pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
 def test_dependent_router_on_calls_of_many_experts(d, E, L, want, flags):
