@@ -153,6 +153,7 @@ __device__ __forceinline__ int union_of_masks(const uint32_t* tm, int L, int wor
   if (threadIdx.x < words) {
     uint32_t un = 0;
     int nact = 0;
+#pragma unroll 1
     for (int t = 0; t < L; ++t) {
       const uint32_t m = tm[threadIdx.x * 32 + t];
       un |= m;
@@ -163,14 +164,17 @@ __device__ __forceinline__ int union_of_masks(const uint32_t* tm, int L, int wor
     um[threadIdx.x] = un;
   }
   __syncthreads();
+#pragma unroll 1
   for (int w = warp; w < words; w += nwarps) {
     int off = 0;
+#pragma unroll 1
     for (int v = 0; v < w; ++v) off += cnt[v];
     const uint32_t un = um[w];
     if ((un >> lane) & 1u) ids_sm[off + __popc(un & ((1u << lane) - 1u))] = 32 * w + lane;
   }
   if (threadIdx.x == 0) {
     int total = 0, total_act = 0;
+#pragma unroll 1
     for (int w = 0; w < words; ++w) {
       total += cnt[w];
       total_act += act[w];
@@ -327,7 +331,9 @@ __device__ __forceinline__ void publish_routing(const RoutingOut& pub, const Rou
   }
   if constexpr (MODE == 2) {      // the scores and masks
     const float* rinv = reinterpret_cast<const float*>(ctl + 104);
+#pragma unroll 1
     for (int t = tid >> 5; pub.scores && t < L; t += blockDim.x >> 5) {
+#pragma unroll 1
       for (int w = 0; w < words; ++w) {
         const int e = 32 * w + lane;
         float sv = 0.0f;
@@ -342,6 +348,7 @@ __device__ __forceinline__ void publish_routing(const RoutingOut& pub, const Rou
       }
     }
   }
+#pragma unroll 1
   for (int e = tid; e < E; e += blockDim.x) {
     if (pub.union_ids) pub.union_ids[e] = e < nu ? ids_sm[e] : -1;
     if (pub.union_mask && e < words) pub.union_mask[e] = (uint32_t)ctl[8 + e];

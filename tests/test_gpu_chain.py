@@ -239,3 +239,50 @@ def test_calls_one_behind_the_other(flags, lengths, d, E):
     torch.cuda.synchronize()
     assert torch.equal(h, want[0]) and torch.equal(x, want[1])
     assert layer.last_status() == 0
+
+
+@pytest.mark.parametrize("d,E,d_e,L", [(192, 24, 64, 1), (1088, 70, 64, 8), (256, 40, 128, 13), (192, 48, 64, 20),
+                                       (512, 100, 256, 6)])
+def test_experts_whose_scores_vanish_are_not_in_the_union(d, E, d_e, L):
+    """gain * ReLU(logit) of every third expert is the smallest denormal number, and 1 / rms takes it
+    to zero; their D is infinite, so that one of them in the union would spoil out."""
+    dw = make(d, E, d_e, 11, 5.0)
+    t, faint = dw.tensors, torch.arange(E, device="cuda") % 3 == 0
+    t["gain"][faint] = 1.4e-45
+    t["W_r"][faint] = 0.0
+    t["bias"][faint] = 0.6                    # one denormal step; rms > 2 makes less than half a step of it
+    t["bias"][1::3] = -9.0                    # never active, by their logits
+    t["D"][faint] = float("inf")
+    x = torch.randn(L, d, device="cuda").bfloat16()
+    clean = dict(t, D=torch.where(faint[:, None, None], 0.0, t["D"].float()).bfloat16())
+    s, ref = reference(clean, x)
+    s[:, faint] = 0.0
+    layer = B.Layer(d, E, d_e, L_max=L)
+    for _ in range(2):
+        r = layer.forward(dw, x)
+        ids = (s != 0).any(0).nonzero().flatten().int()
+        n = int(r.n_union.item())
+        assert n == len(ids) and torch.equal(r.union_ids[:n], ids)
+        assert bool((r.scores[:, faint] == 0).all()) and bool(((r.scores != 0) == (s != 0)).all())
+        assert (r.scores.double() - s).abs().max() <= 1e-5 * max(s.square().mean().sqrt().item(), 1.0)
+        assert (r.out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+    st = layer.stats_host()
+    assert st.n_union == 2 * n and st.n_active == 2 * int((s != 0).sum()) and layer.last_status() == 0
+
+
+@pytest.mark.parametrize("L", [1, 8, 16, 32])
+def test_scores_are_those_of_the_router_kernel_bit_for_bit(L):
+    """Logits that both kernels sum without rounding (small whole numbers): what is left is the sum of
+    squares, its mean, 1 / root and two products."""
+    d, E, d_e = 192, 90, 64
+    layer, dw = B.Layer(d, E, d_e, L_max=L), make(d, E, d_e, 5, 0.0)
+    t = dw.tensors
+    for seed in range(40):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        t["W_r"].copy_(torch.randint(-9, 10, (E, d), device="cuda", generator=g))
+        t["bias"].copy_(torch.randint(-40, 9, (E,), device="cuda", generator=g) / 8)
+        x = torch.randint(-3, 4, (L, d), device="cuda", generator=g).bfloat16()
+        x[:, 8 + seed:] = 0
+        alone = torch.empty(L, E, device="cuda")
+        B.blockffn_router(layer.h, dw.struct, x, L, alone)
+        assert torch.equal(layer.forward(dw, x).scores, alone)
