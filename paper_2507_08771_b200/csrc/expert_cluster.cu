@@ -1055,15 +1055,17 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
 // expected union's U (the hint of the configuration, or 30 % of the experts: the union itself is known on the device
 // only, and a call whose union is another one takes the kernel of the expected one). us per layer of a captured
 // stack, kernel of expert_chain.cu, or with scores given expert_wide.cuh / this one (M elements):
-//   router on, 17 to 32 tokens: below d = 1024 always, above from 24 M elements times tokens. d = 512, E = 16,
-//     d_e = 64 (0.2 M), 17 tokens 11.6 / 11.3; d = 1024, E = 24, d_e = 64 (0.5 M), 24 tokens 11.6 / 12.0; d = 2048, E = 16,
-//     d_e = 64 (0.7 M), 17 tokens 12.8 / 13.4, 32 tokens 13.8 / 13.7; E = 24, d_e = 128 (1.8 M), 17 tokens 13.5 / 13.8,
-//     32 tokens 14.4 / 14.1; d = 1536, E = 48, d_e = 128 (2.8 M), 17 tokens 14.4 / 13.5; d = 2048, E = 128, d_e = 128
-//     (10 M), 32 tokens 24.8 / 18.5
-//   router on, 9 to 16: from 6 M, up to d = 1024 from 9 M. 13 tokens, d = 1792, E = 56, d_e = 128 (3.9 M) 11.9 / 12.6;
-//     d = 2048, E = 64 (5 M) 12 tokens 13.2 / 13.4, 16 tokens 13.7 / 13.5; d = 1536, E = 52, d_e = 256 (6.3 M), 9 tokens
-//     18.4 / 15.4; d = 2048, E = 128 (10 M), 16 tokens 22.2 / 18.5; d = 1024, d_e = 256, E = 80 (6.3 M), 9 tokens 17.2 / 17.9,
-//     E = 100 (7.9 M), 10 tokens 18.9 / 19.4, E = 128 (10 M), 12 tokens 23.1 / 22.9
+//   router on, 17 to 32 tokens: below d = 1024 always, above from 24 M elements times tokens; 9 to 16: from 6 M, up to d = 1024
+//     from 9 M. These two lines are older than the present form of the other kernel, which would put them at the rows of U
+//     that it has room for (16 a CTA with 17 to 32 tokens, 21 with 9 to 16 at d above 1024). They have not been moved: the
+//     kernels round differently, and in a stack whose tokens activate one or two experts each (E = 20, 12 % active) a
+//     logit on the other side of zero changes a token's output as a whole. 17 to 32: d = 256, E = 16, d_e = 64 (307 rows), 17
+//     tokens 9.8 / 11.2; d = 768, E = 48, d_e = 64 (896), 24 tokens 10.5 / 12.3; d = 2048, E = 48, d_e = 128 (1792), 32 tokens
+//     14.2 / 15.0; d = 512, E = 64 (2432), 18 tokens 12.6 / 12.6; d = 1024, E = 64, 32 tokens 14.0 / 13.7; d = 2048, E = 64, 17
+//     and 32 tokens 15.2 / 15.2 and 15.9 / 15.4; d = 1536, E = 128 (4864), 32 tokens 21.4 / 17.2. 9 to 16: d = 2048, E = 64, d_e = 128
+//     (16 rows a CTA), 16 tokens 11.4 / 13.9; d = 1792, E = 80 (21), 16 tokens 14.9 / 14.9; d = 1280, E = 100 (26), 16 tokens
+//     16.0 / 14.3; d = 2048, E = 128, 9 tokens 20.0 / 17.8; d = 1024, E = 100, 16 tokens 12.3 / 13.8; E = 80, d_e = 256 (6.3 M),
+//     9 tokens 15.4 / 16.7; E = 120 (9.4 M), 16 tokens 22.2 / 21.5
 //   scores given, 17 to 32: from 4 M. d = 1536, E = 48 (2.9 M), 18 tokens 11.3 / 11.7; d = 2048, E = 100,
 //     d_e = 64 (3.9 M), 24 tokens 11.2 / 11.5; E = 54, d_e = 128 (4.2 M), 17 tokens 13.1 / 12.4; E = 64 (5 M), 24 tokens
 //     15.7 / 13.2; E = 128 (10 M), 32 tokens 24.2 / 16.9. A list given: from 4.5 M (it is known sooner than a union that
