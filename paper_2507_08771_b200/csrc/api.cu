@@ -29,9 +29,10 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
                                const RoutingOut* pub, const RouterLogits* logits, bool logits_final,
                                cudaStream_t st) {
   // The one-kernel form pays off where calls overlap freely, i.e. where x is stable (for a
-  // router-on call: the router has finished before the expert stage starts). A call of up to 8
-  // tokens in a dependent chain (x comes from the call before) runs as the pair, whose two
-  // hand-overs are shorter than a grid-wide exchange inside one kernel. A longer chunk is one kernel, which
+  // router-on call: the router has finished before the expert stage starts). A call of up to 16 tokens in a
+  // dependent chain (x comes from the call before) with stable scores is one kernel made for that where its share
+  // of the union is small (expert_chain_supported has the figures); else one of up to 8 tokens runs as the pair,
+  // whose D is fetched under its up projection. A longer chunk is one kernel, which
   // reads its weights once for all tokens, where the pair reads what shared memory does not hold once per 8:
   // on clusters where the union is large (expert_cluster_supported has the figures), else the one-kernel form
   // on the whole device. Without a promise either is launched cooperatively. List given, nothing promised, us
@@ -47,6 +48,8 @@ cudaError_t launch_tensor_core(blockffn_ctx* c, const blockffn_weights* w, const
     if (e != cudaErrorCooperativeLaunchTooLarge) return e;
     cudaGetLastError();          // (a context with fewer SMs than the device)
   }
+  if (!x_stable && !logits && !union_ids && (call_flags & BLOCKFFN_CALL_INDEPENDENT) && expert_chain_supported(c, L, 0))
+    return launch_expert_chain(c, w, x, scores, L, out, x_next, call_flags, pub, st);
   if ((x_stable || dep_long || dep_inside) &&
       expert_lean_supported(c, L, logits != nullptr, x_stable, logits && logits->a0 == nullptr)) {
     const cudaError_t e = launch_expert_lean(c, w, x, scores, L, union_ids, n_union, out, x_next,
@@ -319,9 +322,9 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
                  ? BLOCKFFN_OK
                  : BLOCKFFN_ERR_CUDA;
     }
-    if (!x_stable_call && expert_chain_supported(h, L)) {
+    if (!x_stable_call && expert_chain_supported(h, L, 3)) {
       h->last_layer_waited_first = false;
-      return launch_expert_chain(h, w, x, L, out, x_next, call_flags, &pub_in, st) == cudaSuccess
+      return launch_expert_chain(h, w, x, nullptr, L, out, x_next, call_flags, &pub_in, st) == cudaSuccess
                  ? BLOCKFFN_OK
                  : BLOCKFFN_ERR_CUDA;
     }

@@ -127,8 +127,9 @@ cudaError_t launch_expert_lean(blockffn_ctx* c, const blockffn_weights* w, const
                                const RoutingOut* pub, const RouterLogits* logits, bool logits_final,
                                cudaStream_t st);
 
-// A whole layer call, router inside, in a dependent chain as one kernel (expert_chain.cu).
-bool expert_chain_supported(const blockffn_ctx* c, int L);
+// A whole layer call in a dependent chain as one kernel (expert_chain.cu): the router inside (scores == NULL, mode 3),
+// or scores given that are promised stable (mode 0).
+bool expert_chain_supported(const blockffn_ctx* c, int L, int mode);
 size_t expert_chain_ws_bytes(const blockffn_config* cfg, int sms);
 cudaError_t expert_chain_setup(blockffn_ctx* c);
 // What is in chain_ws: both kernels of dependent calls work on it and count calls in the same way.
@@ -141,8 +142,8 @@ struct ChainWorkspace {
   size_t h_slot;
 };
 ChainWorkspace chain_workspace(const blockffn_ctx* c);
-cudaError_t launch_expert_chain(blockffn_ctx* c, const blockffn_weights* w, const void* x, int L,
-                                float* out, void* x_next, int call_flags, const RoutingOut* pub,
+cudaError_t launch_expert_chain(blockffn_ctx* c, const blockffn_weights* w, const void* x,
+                                const float* scores, int L, float* out, void* x_next, int call_flags, const RoutingOut* pub,
                                 cudaStream_t st);
 
 // Elements of U of the experts that the caller expects in a chunk's union (by default 30 % of all).

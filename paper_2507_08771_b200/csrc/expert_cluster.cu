@@ -1081,7 +1081,7 @@ ClusterPlan cluster_plan(const blockffn_ctx* c, int L, int mode) {
   const long long u = expected_union_elements(c);
   const int d = c->cfg.d;
   if (L > 16 && L <= 32) {
-    if (mode == 3 ? d >= 1024 && u * L < 24000000 && expert_chain_supported(c, L) : u < (mode == 1 ? 4500000 : 4000000))
+    if (mode == 3 ? d >= 1024 && u * L < 24000000 && expert_chain_supported(c, L, 3) : u < (mode == 1 ? 4500000 : 4000000))
       return ClusterPlan{};
     return cluster_plan_of<4>(c->cfg, L, c->clusters);
   }

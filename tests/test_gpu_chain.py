@@ -286,3 +286,56 @@ def test_scores_are_those_of_the_router_kernel_bit_for_bit(L):
         alone = torch.empty(L, E, device="cuda")
         B.blockffn_router(layer.h, dw.struct, x, L, alone)
         assert torch.equal(layer.forward(dw, x).scores, alone)
+
+
+@pytest.mark.parametrize("d,E,d_e,L", [(320, 90, 128, 8), (1024, 130, 64, 3), (960, 90, 256, 6), (1088, 60, 64, 1),
+                                       (2048, 40, 128, 7), (64, 5, 64, 16), (512, 40, 64, 13), (2048, 70, 128, 16),
+                                       (1792, 33, 64, 9)])
+def test_scores_given(d, E, d_e, L):
+    """Scores that are stable, x from the call before: some, all and none of the experts, a token that is not finite,
+    then a sequence of layers whose x is what the call before left, against the kernels of other handles."""
+    layer, plain = B.Layer(d, E, d_e, L_max=L), B.Layer(d, E, d_e, L_max=L, flags=B.CFG_TWO_KERNELS)
+    dw = make(d, E, d_e, 5, 0.0)
+    t, g = dw.tensors, torch.Generator(device="cuda").manual_seed(d + L)
+    F = B.CALL_INDEPENDENT | B.CALL_ACCUMULATE
+    for k, (u, nan) in enumerate(((max(1, E * 3 // 10), False), (E, False), (0, False), (max(1, E // 4), True))):
+        pick = torch.randperm(E, device="cuda", generator=g)[:u].sort().values.int()
+        s = torch.zeros(L, E, device="cuda")
+        s[:, pick.long()] = (torch.rand(L, u, device="cuda", generator=g) < 0.5) * 0.5 + 0.25
+        if L > 1:
+            s[0] = 0                                   # a token without experts
+        x = torch.randn(L, d, device="cuda", generator=g).bfloat16()
+        if k % 2:                                      # 16-byte but not 32-byte aligned
+            x = torch.cat([x.new_zeros(8), x.flatten()])[8:].view(L, d)
+        if nan:
+            x[L - 1, 3] = float("nan")
+        z = torch.einsum("ejd,td->tej", t["U"].double(), x.double())
+        ref = torch.einsum("tej,ecj->tc", s.double()[:, :, None] * z * torch.sigmoid(z), t["D"].double())
+        base = torch.randn(L, d, device="cuda", generator=g)
+        out, nxt = base.clone(), torch.empty(L, d, dtype=torch.bfloat16, device="cuda")
+        torch.cuda.synchronize()
+        n0 = layer.launch_count()
+        r = layer.forward_scores(dw, x, s, out=out, x_next=nxt, call_flags=F)
+        assert layer.launch_count() - n0 == 2           # one kernel, and the copies of the routing
+        ids = (s != 0).any(0).nonzero().flatten().int()
+        n = int(r.n_union.item())
+        assert n == len(ids) and torch.equal(r.union_ids[:n], ids) and layer.last_status() == 0
+        rows = L - 1 if nan else L
+        rms = max(ref[:rows].square().mean().sqrt().item(), 1e-6) if rows else 1.0
+        assert rows == 0 or (out[:rows].double() - base[:rows].double() - ref[:rows]).abs().max().item() <= 2e-2 * rms + 1e-6
+        assert torch.equal(nxt[:rows], out[:rows].bfloat16())
+        if nan:
+            assert bool(out[L - 1].isnan().all())
+    ss = [torch.where(torch.rand(L, E, device="cuda", generator=g) < 0.2, 1.0 / E, 0.0) for _ in range(3)]   # (h keeps its scale)
+    x0 = torch.randn(L, d, device="cuda", generator=g).bfloat16()
+    got = []
+    for handle in (layer, plain):
+        h, xs = x0.float(), [x0.clone(), torch.empty_like(x0)]
+        torch.cuda.synchronize()
+        for i in range(24):
+            B.blockffn_layer_forward_scores(handle.h, dw.struct, xs[i % 2], ss[i % 3], L, h, xs[(i + 1) % 2],
+                                            handle.stats, F)
+        got.append(h.clone())
+        assert handle.last_status() == 0
+    # (what the 24 layers add is about as large as x; sums in another order move some of their bf16 x and h by a step, 2^-8)
+    assert (got[0] - got[1]).abs().max() <= 2e-2 * got[1].square().mean().sqrt()
