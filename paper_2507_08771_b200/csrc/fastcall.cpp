@@ -161,8 +161,36 @@ PyObject* reuse_ratio(PyObject*, PyObject* const* a, Py_ssize_t n) {
   });
 }
 
-// What Layer.forward returns beside out: scores [L][E] and tok_mask [L][words] (or None, None),
-// union_mask [words], union_ids [E], n_union [1] on CUDA device `index` (-1: the current one).
+// scores [L][E] and tok_mask [L][words] (where with_scores), union_mask [words], union_ids [E], n_union [1] on CUDA
+// device `index` (-1: the current one)
+struct Routing {
+  at::Tensor b[5];
+  Routing(int64_t L, int64_t E, int64_t words, int with_scores, int index) {
+    const auto dev = at::device(at::Device(at::kCUDA, static_cast<c10::DeviceIndex>(index)));
+    const auto i32 = dev.dtype(at::kInt);
+    if (with_scores) {
+      b[0] = at::empty({L, E}, dev.dtype(at::kFloat));
+      b[1] = at::empty({L, words}, i32);
+    }
+    b[2] = at::empty({words}, i32);
+    b[3] = at::empty({E}, i32);
+    b[4] = at::empty({1}, i32);
+  }
+};
+// t[at ..]: the tensors, None where there is none. False with an error set, and t gone, when that fails.
+bool put(PyObject*& t, int at, const at::Tensor* b, int n) {
+  for (int k = 0; t && k < n; ++k) {
+    PyObject* o = b[k].defined() ? THPVariable_Wrap(b[k]) : Py_NewRef(Py_None);
+    if (o) {
+      PyTuple_SET_ITEM(t, at + k, o);
+    } else {
+      Py_CLEAR(t);
+    }
+  }
+  return t != nullptr;
+}
+
+// What Layer.forward returns beside out
 PyObject* routing_buffers(PyObject*, PyObject* const* a, Py_ssize_t n) {
   if (n != 5) {
     PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
@@ -173,28 +201,66 @@ PyObject* routing_buffers(PyObject*, PyObject* const* a, Py_ssize_t n) {
   const int with_scores = g.number(3), index = g.number(4);
   if (!g.ok) Py_RETURN_NOTIMPLEMENTED;
   try {
-    const auto dev = at::device(at::Device(at::kCUDA, static_cast<c10::DeviceIndex>(index)));
-    const auto i32 = dev.dtype(at::kInt);
-    at::Tensor b[5];               // (all of them exist before the first becomes a Python object)
-    if (with_scores) {
-      b[0] = at::empty({L, E}, dev.dtype(at::kFloat));
-      b[1] = at::empty({L, words}, i32);
-    }
-    b[2] = at::empty({words}, i32);
-    b[3] = at::empty({E}, i32);
-    b[4] = at::empty({1}, i32);
+    const Routing r(L, E, words, with_scores, index);   // (all of them exist before the first becomes a Python object)
     PyObject* t = PyTuple_New(5);
-    for (int k = 0; t && k < 5; ++k) {
-      PyObject* o = b[k].defined() ? THPVariable_Wrap(b[k]) : Py_NewRef(Py_None);
+    put(t, 0, r.b, 5);
+    return t;
+  } catch (const std::exception&) {
+    Py_RETURN_NOTIMPLEMENTED;
+  }
+}
+
+// Layer.forward with nothing given but x: out and the routing buffers, blockffn_layer_forward and
+// blockffn_read_routing on the current stream, (status, status, out, the buffers).
+// (handle, weights, x, x_next, stats, call_flags, d, E, words, device index)
+PyObject* layer_call(PyObject*, PyObject* const* a, Py_ssize_t n) {
+  if (n != 10) {
+    PyErr_SetString(PyExc_TypeError, "wrong number of arguments");
+    return nullptr;
+  }
+  bool launched = false;
+  try {
+    Args g{a};
+    const blockffn_handle h = g.handle(0);
+    const blockffn_weights* w = g.weights(1);
+    const void* x = g.device<void>(2);
+    void* xn = g.device<void>(3);
+    blockffn_stats* stats = g.device<blockffn_stats>(4);
+    const int fl = g.number(5), index = g.number(9);
+    const int64_t d = g.number(6), E = g.number(7), words = g.number(8);
+    if (!g.ok || !x || THPVariable_Unpack(a[2]).dim() < 1) Py_RETURN_NOTIMPLEMENTED;
+    const int64_t L = THPVariable_Unpack(a[2]).size(0);
+    if (L > (1 << 20)) Py_RETURN_NOTIMPLEMENTED;       // (refused below; not by running out of memory here)
+    const at::Tensor out =
+        at::empty({L, d}, at::device(at::Device(at::kCUDA, static_cast<c10::DeviceIndex>(index))).dtype(at::kFloat));
+    const Routing r(L, E, words, 1, index);
+    void* st = c10::cuda::getCurrentCUDAStream().stream();
+    int code[2];
+    launched = true;
+    Py_BEGIN_ALLOW_THREADS
+    code[0] = blockffn_layer_forward(h, w, x, static_cast<int32_t>(L), out.data_ptr<float>(), xn, stats, fl, st);
+    code[1] = code[0] != BLOCKFFN_OK
+                  ? BLOCKFFN_OK
+                  : blockffn_read_routing(h, static_cast<int32_t>(L), r.b[0].data_ptr<float>(),
+                                          reinterpret_cast<uint32_t*>(r.b[1].data_ptr<int32_t>()),
+                                          reinterpret_cast<uint32_t*>(r.b[2].data_ptr<int32_t>()),
+                                          r.b[3].data_ptr<int32_t>(), r.b[4].data_ptr<int32_t>(), st);
+    Py_END_ALLOW_THREADS
+    PyObject* t = PyTuple_New(8);
+    for (int k = 0; t && k < 2; ++k) {
+      PyObject* o = PyLong_FromLong(code[k]);
       if (o) {
         PyTuple_SET_ITEM(t, k, o);
       } else {
         Py_CLEAR(t);
       }
     }
+    if (t && put(t, 2, &out, 1)) put(t, 3, r.b, 5);
     return t;
-  } catch (const std::exception&) {
-    Py_RETURN_NOTIMPLEMENTED;
+  } catch (const std::exception& e) {
+    if (!launched) Py_RETURN_NOTIMPLEMENTED;
+    if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, e.what());
+    return nullptr;
   }
 }
 
@@ -226,6 +292,7 @@ PyMethodDef g_methods[] = {
     method<read_routing>("read_routing"),
     method<reuse_ratio>("reuse_ratio"),
     method<routing_buffers>("routing_buffers"),
+    method<layer_call>("layer_call"),
     method<set_types>("set_types"),
     {nullptr, nullptr, 0, nullptr},
 };

@@ -22,6 +22,18 @@ def test_what_is_not_plain_is_left_to_ctypes():
         fast.layer_forward(h)
 
 
+def test_a_layer_call_that_is_not_plain_is_left_to_its_parts():
+    fast = B._load_fast()
+    h, w, t = ctypes.c_void_p(0), B.make_weights(), torch.zeros(8)
+    plain = [h, w, t, None, None, 0, 8, 4, 1, 1 << 6]      # (a tensor that is not on a GPU, a device that does not exist)
+    for i, odd in [(0, None), (1, None), (2, None), (2, 64), (2, t), (3, t), (5, None), (6, 1.0), (9, None)]:
+        args = list(plain)
+        args[i] = odd
+        assert fast.layer_call(*args) is NotImplemented, (i, odd)
+    with pytest.raises(TypeError):
+        fast.layer_call(h)
+
+
 def test_buffers_that_cannot_be_allocated_leave_nothing_behind():
     fast = B._load_fast()
     args = (1 << 30, 1 << 30, 1 << 30, 0, 1 << 6)      # a device that does not exist
@@ -95,3 +107,23 @@ def test_both_ways_give_the_same():
     assert [tuple(b.shape) for b in bufs] == [(L, E), (L, 2), (2,), (E,), (1,)]
     assert [b.dtype for b in bufs] == [torch.float32] + 4 * [torch.int32]
     assert [b is None for b in layer._routing(L, False)] == [True, True, False, False, False]
+
+
+@pytest.mark.gpu
+def test_a_layer_call_at_once_is_the_call_in_its_parts():
+    layer = B.Layer(256, 16, 64, L_max=8)
+    g = torch.Generator(device="cuda").manual_seed(1)
+    t = {"W_r": (256 ** -0.5 * torch.randn(16, 256, device="cuda", generator=g)).bfloat16(), "gain": torch.ones(16, device="cuda"),
+         "U": torch.randn(16, 64, 256, device="cuda", generator=g).bfloat16(),
+         "D": torch.randn(16, 256, 64, device="cuda", generator=g).bfloat16()}
+    dw = B.DeviceWeights(B.make_weights(t["W_r"], t["gain"], None, t["U"], t["D"]), t)
+    for L in (1, 5, 8):
+        x, nxt = torch.randn(L, 256, device="cuda", generator=g).bfloat16(), [torch.empty(L, 256, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        a = layer.forward(dw, x, x_next=nxt[0])
+        b = layer.forward(dw, x, out=torch.empty(L, 256, device="cuda"), x_next=nxt[1])
+        for u, v in zip((a.out, a.scores, a.tok_mask, a.union_mask, a.n_union, nxt[0]), (b.out, b.scores, b.tok_mask, b.union_mask, b.n_union, nxt[1])):
+            assert u.shape == v.shape and u.dtype == v.dtype and torch.equal(u, v)
+        assert torch.equal(a.union_ids, b.union_ids)
+    with pytest.raises(B.BlockFFNError) as e:
+        layer.forward(dw, torch.zeros(9, 256, dtype=torch.bfloat16, device="cuda"))       # more than L_max
+    assert e.value.code == B.ERR_INVALID_ARG and "blockffn_layer_forward" in str(e.value)
