@@ -126,6 +126,31 @@ def test_calls_after_one_whose_wait_ran_out(held, L):
     cfg.flags = 0
 
 
+@pytest.mark.parametrize("L", [4, 12, 24])
+@pytest.mark.parametrize("E", [70, 130])
+def test_a_wait_that_runs_out_before_the_last_experts(E, L):
+    """More experts than are looked at in one trip (64): the first trip's logits do not come within the limit, and those
+    behind it are there at a second look. The call gives up all the same, and the next ones find everything in order."""
+    d, d_e = 192, 64
+    dw, layer = make(d, E, d_e, 7, -0.5), B.Layer(d, E, d_e, L_max=32)
+    cfg = B.Config.from_address(layer.h.value)       # the handle begins with its configuration
+    assert (cfg.d, cfg.E, cfg.d_e, cfg.L_max, cfg.flags) == (d, E, d_e, 32, 0)
+    for k in range(2):                               # (either of the two buffers of h)
+        for n in [L] * (k + 1) + [0] + [L, 32, 1, L]:
+            cfg.flags = 0 if n else B.CFG_TEST_EXPIRE_WAIT
+            x = torch.randn(n or L, d, device="cuda").bfloat16()
+            out = torch.full((n or L, d), 7.0, device="cuda")
+            B.blockffn_layer_forward(layer.h, dw.struct, x, n or L, out)
+            if n:
+                _, ref = reference(dw.tensors, x)
+                assert layer.last_status() == 0
+                assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+            else:
+                assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+                assert bool((out == 7.0).all())
+    cfg.flags = 0
+
+
 def test_a_new_handle_has_its_workspace_filled():
     """The first call may come on a stream that is not ordered behind the default one, where
     blockffn_create fills the workspace (250 MB of "not written yet" here, some 40 us of work)."""
