@@ -315,7 +315,8 @@ def test_scores_are_those_of_the_router_kernel_bit_for_bit(L):
 
 @pytest.mark.parametrize("d,E,d_e,L", [(320, 90, 128, 8), (1024, 130, 64, 3), (960, 90, 256, 6), (1088, 60, 64, 1),
                                        (2048, 40, 128, 7), (64, 5, 64, 16), (512, 40, 64, 13), (2048, 70, 128, 16),
-                                       (1792, 33, 64, 9)])
+                                       (1792, 33, 64, 9), (448, 250, 64, 7), (320, 200, 64, 14), (512, 64, 128, 2),
+                                       (256, 65, 128, 15), (1088, 64, 64, 16)])
 def test_scores_given(d, E, d_e, L):
     """Scores that are stable, x from the call before: some, all and none of the experts, a token that is not finite,
     then a sequence of layers whose x is what the call before left, against the kernels of other handles."""
