@@ -267,7 +267,7 @@ def test_calls_one_behind_the_other(flags, lengths, d, E):
 
 
 @pytest.mark.parametrize("d,E,d_e,L", [(192, 24, 64, 1), (1088, 70, 64, 8), (256, 40, 128, 13), (192, 48, 64, 20),
-                                       (512, 100, 256, 6)])
+                                       (512, 100, 256, 6), (256, 150, 64, 5), (1088, 140, 64, 12), (192, 300, 64, 20)])
 def test_experts_whose_scores_vanish_are_not_in_the_union(d, E, d_e, L):
     """gain * ReLU(logit) of every third expert is the smallest denormal number, and 1 / rms takes it
     to zero; their D is infinite, so that one of them in the union would spoil out."""
@@ -295,11 +295,12 @@ def test_experts_whose_scores_vanish_are_not_in_the_union(d, E, d_e, L):
     assert st.n_union == 2 * n and st.n_active == 2 * int((s != 0).sum()) and layer.last_status() == 0
 
 
+@pytest.mark.parametrize("E", [90, 129, 200])
 @pytest.mark.parametrize("L", [1, 8, 16, 32])
-def test_scores_are_those_of_the_router_kernel_bit_for_bit(L):
+def test_scores_are_those_of_the_router_kernel_bit_for_bit(L, E):
     """Logits that both kernels sum without rounding (small whole numbers): what is left is the sum of
     squares, its mean, 1 / root and two products."""
-    d, E, d_e = 192, 90, 64
+    d, d_e = 192, 64
     layer, dw = B.Layer(d, E, d_e, L_max=L), make(d, E, d_e, 5, 0.0)
     t = dw.tensors
     for seed in range(40):
@@ -311,6 +312,22 @@ def test_scores_are_those_of_the_router_kernel_bit_for_bit(L):
         alone = torch.empty(L, E, device="cuda")
         B.blockffn_router(layer.h, dw.struct, x, L, alone)
         assert torch.equal(layer.forward(dw, x).scores, alone)
+
+
+@pytest.mark.parametrize("d,E,d_e", [(64, 129, 64), (192, 160, 64), (256, 257, 64), (1088, 257, 64), (320, 1024, 64)])
+def test_many_experts(d, E, d_e):
+    """More than 128 experts: edges of the words of a mask and of a trip through the logits, unions of some, few and all."""
+    layer, lengths = B.Layer(d, E, d_e, L_max=32), (1, 8, 9, 16, 17, 32)
+    for seed, bias in enumerate((-0.5, 0.5, 9.0)):
+        dw = make(d, E, d_e, seed, bias)
+        t = dw.tensors
+        t["bias"][32:64] = -9.0                        # a word of the masks without experts
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        for L in lengths:
+            check(layer, dw, torch.randn(L, d, device="cuda", generator=g).bfloat16(), B.CALL_INDEPENDENT)
+    assert layer.last_status() == 0
+    st = layer.stats_host()
+    assert st.n_chunks == 3 * len(lengths) and st.n_tokens == 3 * sum(lengths)
 
 
 @pytest.mark.parametrize("d,E,d_e,L", [(320, 90, 128, 8), (1024, 130, 64, 3), (960, 90, 256, 6), (1088, 60, 64, 1),
