@@ -51,7 +51,7 @@ def check(layer, dw, x, flags):
     assert torch.equal(bits.bool(), active)
 
 
-@pytest.mark.parametrize("d,E,d_e", [(64, 5, 64), (320, 33, 64), (1024, 16, 256), (1088, 130, 64), (2048, 64, 128)])
+@pytest.mark.parametrize("d,E,d_e", [(64, 5, 64), (320, 33, 64), (1024, 16, 256), (1088, 130, 64), (2048, 64, 128), (1536, 60, 256)])
 @pytest.mark.parametrize("flags", [0, B.CALL_INDEPENDENT])
 def test_chunk_lengths_and_unions_on_one_handle(d, E, d_e, flags):
     layer = B.Layer(d, E, d_e, L_max=32)
