@@ -188,8 +188,8 @@ def chain(layer, dws, lengths, h, x, flags, each=lambda i: None):
 
 @pytest.mark.parametrize("d,E,d_e", [(64, 40, 64), (128, 64, 64), (192, 128, 128), (192, 24, 256), (1984, 16, 64), (1024, 31, 64)])
 def test_long_chunks_off_the_clusters(d, E, d_e):
-    """17 to 32 tokens at widths or expected unions too small for the clusters, and the same from a handle that expects so few
-    experts that the throughput kernel takes them: one by one, one behind the other, and with a wait that runs out."""
+    """17 to 32 tokens at widths or expected unions too small for the clusters, from a handle with the usual expectation and from
+    one that expects a single expert: one by one, one behind the other, and with a wait that runs out."""
     # (At -0.5 a third of the experts is active, and the RMS of a token's logits is 0.1 or more: their error, up to
     # 1e-6, is then within 1e-5 of a score. At -1.6 some tokens have one active logit of a few thousandths, and
     # 1e-6 of it is 1e-4 of its score: 5e-5 seen, with the 1e-5 of check missed.)
@@ -382,3 +382,95 @@ def test_scores_given(d, E, d_e, L):
         assert handle.last_status() == 0
     # (what the 24 layers add is about as large as x; sums in another order move some of their bf16 x and h by a step, 2^-8)
     assert (got[0] - got[1]).abs().max() <= 2e-2 * got[1].square().mean().sqrt()
+
+
+def scores_like(L, E, g, share=0.3):
+    s = torch.rand(L, E, device="cuda", generator=g)
+    return torch.where(s < share, s + 0.1, 0.0)
+
+
+@pytest.mark.parametrize("L", [1, 8, 14])
+def test_calls_after_one_whose_wait_ran_out_scores_given(L):
+    """As above, with scores given: the wait for h. The calls around it are of both kinds."""
+    d, E, d_e = 512, 64, 128
+    dw, layer = make(d, E, d_e, 7, -0.5), B.Layer(d, E, d_e, L_max=16)
+    g = torch.Generator(device="cuda").manual_seed(L)
+    cfg = B.Config.from_address(layer.h.value)       # the handle begins with its configuration
+    assert (cfg.d, cfg.E, cfg.d_e, cfg.L_max, cfg.flags) == (d, E, d_e, 16, 0)
+    for k in range(2):                               # (either of the two buffers of h)
+        for n in [L] * (k + 1) + [0] + [L, -16, 1, -1, L]:      # (0: held; negative: router on)
+            cfg.flags = 0 if n else B.CFG_TEST_EXPIRE_WAIT
+            T = abs(n) or L
+            x, s = torch.randn(T, d, device="cuda", generator=g).bfloat16(), scores_like(T, E, g)
+            s[0, ::5] = 0.5
+            out = torch.full((T, d), 7.0, device="cuda")
+            torch.cuda.synchronize()
+            n0 = layer.launch_count()
+            if n < 0:
+                B.blockffn_layer_forward(layer.h, dw.struct, x, T, out)
+                _, ref = reference(dw.tensors, x)
+            else:
+                B.blockffn_layer_forward_scores(layer.h, dw.struct, x, s, T, out, call_flags=B.CALL_INDEPENDENT)
+                z = torch.einsum("ejd,td->tej", dw.tensors["U"].double(), x.double())
+                ref = torch.einsum("tej,ecj->tc", s.double()[:, :, None] * z * torch.sigmoid(z), dw.tensors["D"].double())
+            assert layer.launch_count() - n0 == 1
+            if n:
+                assert layer.last_status() == 0
+                assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
+            else:
+                assert layer.last_status(clear=True) == B.DEV_WAIT_EXPIRED
+                assert bool((out == 7.0).all())
+    cfg.flags = 0
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_scores_given_in_turn_with_other_calls(graph):
+    """Scores given, router on and clusters on one handle, every x from the call before: they share tickets and both
+    buffers of h. The same bits as with a pause behind every call, eagerly or from a graph, alone and beside another
+    handle's calls on another stream."""
+    d, E, d_e, N = 1024, 64, 128, 24
+    dws = [make(d, E, d_e, s, b) for s, b in enumerate((-0.5, 0.3, -1.0))]
+    for dw in dws:
+        dw.tensors["D"].mul_(1.0 / E)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    scores = [scores_like(16, E, g) for _ in range(4)]
+    lengths = [(8, True), (5, False), (16, True), (32, False), (13, True), (16, False), (1, True), (24, False), (8, True), (8, True)]
+    start = torch.randn(32, d, device="cuda", generator=g)
+    layers = [B.Layer(d, E, d_e, L_max=32) for _ in range(2)]
+    hs = [start.clone() for _ in range(2)]
+    xs = [torch.zeros(2, 32, d, dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+
+    def run(k, each=lambda: None):
+        h, x, layer = hs[k], xs[k], layers[k]
+        h.copy_(start)
+        x.copy_(start.expand(2, 32, d))
+        for i in range(N):
+            L, given = lengths[i % len(lengths)]
+            F, w = B.CALL_INDEPENDENT | B.CALL_ACCUMULATE, dws[i % 3].struct
+            if given:
+                B.blockffn_layer_forward_scores(layer.h, w, x[i % 2], scores[i % 4], L, h, x[(i + 1) % 2], None, F)
+            else:
+                B.blockffn_layer_forward(layer.h, w, x[i % 2], L, h, x[(i + 1) % 2], None, F)
+            each()
+
+    torch.cuda.synchronize()
+    n0 = layers[0].launch_count()
+    run(0, torch.cuda.synchronize)
+    assert layers[0].launch_count() - n0 == N
+    want = hs[0].clone()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    graphs = []
+    for k in range(2):
+        if graph:
+            graphs.append(torch.cuda.CUDAGraph())
+            with torch.cuda.graph(graphs[k], stream=streams[k]):
+                run(k)
+    for both in (False, True):
+        torch.cuda.synchronize()
+        for _ in range(4):
+            for k in range(1 + both):
+                with torch.cuda.stream(streams[k]):
+                    graphs[k].replay() if graph else run(k)
+        torch.cuda.synchronize()
+        for k in range(1 + both):
+            assert layers[k].last_status() == 0 and torch.equal(hs[k], want)
