@@ -29,12 +29,13 @@
  *     never fault; read it with blockffn_last_status().
  *   - Calls whose CTAs exchange data inside one kernel need all CTAs of the call resident at
  *     once, at most one per SM: blockffn_layer_forward, and scores-in or list calls with one of
- *     the two promises below (the INDEPENDENT flags). Such calls of two handles on two streams
+ *     the two promises below (the INDEPENDENT flags), of any length. They are sized for the device, so
+ *     a context with fewer SMs has no room for them. Such calls of two handles on two streams
  *     are fine while other work lets go of the SMs in time; a call that cannot get its SMs
  *     within a second gives up (BLOCKFFN_DEV_WAIT_EXPIRED). (Longer dependent chunks run on clusters
  *     of four CTAs: those need their four SMs from one group of SMs, all four at a time.) A program that shares the GPU with
- *     kernels that hold SMs for that long, or that runs several handles' calls at the same time
- *     on streams of different priorities, sets BLOCKFFN_CFG_TWO_KERNELS: no kernel then waits
+ *     kernels that hold SMs for that long, that gives it a part of the SMs only, or that runs several
+ *     handles' calls at the same time on streams of different priorities, sets BLOCKFFN_CFG_TWO_KERNELS: no kernel then waits
  *     for another CTA. Scores-in and list calls without a promise do not have that condition: of
  *     more than 8 tokens they are launched cooperatively, i.e. start when all their CTAs fit.
  *   - Limits: 1 <= L <= L_max <= 32 per call; d % 8 == 0; d_e % 8 == 0;
@@ -100,8 +101,9 @@ typedef struct {
  * weights while the kernel enqueued before it on the stream is still finishing
  * (programmatic dependent launch); this bit launches them fully serialised instead. */
 #define BLOCKFFN_CFG_NO_CHAINING 0x10000
-/* A call whose x is stable, a router-on layer call and a chunk of more than 8 tokens normally run
- * as one kernel whose CTAs exchange the intermediate (and the router's logits); this bit selects
+/* A call whose x is stable, a router-on layer call, a scores-in layer call whose scores are promised
+ * stable and a chunk of more than 8 tokens normally run (most shapes) as one kernel whose CTAs
+ * exchange the intermediate (and the router's logits); this bit selects
  * kernels that follow one another instead (router, up projection, down projection) for all of
  * them. Same results within the tolerance. For programs that share the GPU, see the
  * conventions above, and for comparison.                                                    */

@@ -332,8 +332,9 @@ blockffn_status blockffn_layer_forward(blockffn_handle h, const blockffn_weights
       // x stable: the router runs inside the one-kernel form (its CTAs share the experts' logits
       // out between them and exchange them through L2), so the call is one launch that overlaps
       // its neighbours like a scores-in call. A dependent call of more than 8 tokens comes here where
-      // neither kernel above takes it: a score matrix too large for the chain kernel's pools where the
-      // clusters do not take the shape. One launch on the whole device.
+      // neither kernel above takes it: a score matrix too large for the chain kernel's pools (d above 1024 and
+      // 875 experts and more at 32 tokens) where the clusters do not take the shape either, which they do wherever
+      // the device holds the usual number of them. One launch on the whole device.
       const RouterLogits lg_in{nullptr, router_gain(h, w), h->cfg.rms_eps};
       h->last_layer_waited_first = false;
       return launch_tensor_core(h, w, x, h->scores, L, nullptr, nullptr, out, x_next, flags, &pub_in,

@@ -136,7 +136,9 @@ cudaError_t expert_chain_setup(blockffn_ctx* c);
 struct ChainWorkspace {
   unsigned long long* seq;      // tickets, num_sms per call
   uint32_t* used;               // [2] 16-byte pieces of each h buffer that its last call wrote
-  unsigned long long* logits;   // copies of [L][E] words {logit, call number}
+  unsigned long long* logits;   // copies of the words {logit, call number}: [E][8, 16 or 32 tokens] in expert_chain.cu, [L][E] in
+                                // expert_cluster.cu. A word counts only with the number of the call that looks at it, and the
+                                // two count calls together, so that neither takes the other's words for its own.
   size_t logit_copy;            // words from one copy to the next
   uint16_t* h;                  // two buffers of h_slot elements
   size_t h_slot;

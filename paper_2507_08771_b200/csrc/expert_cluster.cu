@@ -1060,9 +1060,9 @@ ClusterPlan cluster_plan_of(const blockffn_config& cfg, int L, int clusters) {
 //     that it has room for (16 a CTA with 17 to 32 tokens, 21 with 9 to 16 at d above 1024). They have not been moved: the
 //     kernels round differently, and in a stack whose tokens activate one or two experts each (E = 20, 12 % active) a
 //     logit on the other side of zero changes a token's output as a whole. 17 to 32: d = 256, E = 16, d_e = 64 (307 rows), 17
-//     tokens 9.8 / 11.2; d = 768, E = 48, d_e = 64 (896), 24 tokens 10.5 / 12.3; d = 2048, E = 48, d_e = 128 (1792), 32 tokens
-//     14.2 / 15.0; d = 512, E = 64 (2432), 18 tokens 12.6 / 12.6; d = 1024, E = 64, 32 tokens 14.0 / 13.7; d = 2048, E = 64, 17
-//     and 32 tokens 15.2 / 15.2 and 15.9 / 15.4; d = 1536, E = 128 (4864), 32 tokens 21.4 / 17.2. 9 to 16: d = 2048, E = 64, d_e = 128
+//     tokens 8.8 / 11.0; d = 768, E = 48, d_e = 64 (896), 24 tokens 10.3 / 12.2; d = 2048, E = 48, d_e = 128 (1792), 32 tokens
+//     13.4 / 14.7; d = 512, E = 64 (2432), 18 tokens 12.9 / 12.6; d = 1024, E = 64, 32 tokens 14.6 / 13.6; d = 2048, E = 64, 17
+//     and 32 tokens 15.3 / 15.1 and 16.2 / 15.4; d = 1536, E = 128 (4864), 32 tokens 21.3 / 17.0. 9 to 16: d = 2048, E = 64, d_e = 128
 //     (16 rows a CTA), 16 tokens 11.4 / 13.9; d = 1792, E = 80 (21), 16 tokens 14.9 / 14.9; d = 1280, E = 100 (26), 16 tokens
 //     16.0 / 14.3; d = 2048, E = 128, 9 tokens 20.0 / 17.8; d = 1024, E = 100, 16 tokens 12.3 / 13.8; E = 80, d_e = 256 (6.3 M),
 //     9 tokens 15.4 / 16.7; E = 120 (9.4 M), 16 tokens 22.2 / 21.5
