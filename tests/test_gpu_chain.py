@@ -474,3 +474,20 @@ def test_scores_given_in_turn_with_other_calls(graph):
         torch.cuda.synchronize()
         for k in range(1 + both):
             assert layers[k].last_status() == 0 and torch.equal(hs[k], want)
+
+
+@pytest.mark.parametrize("u,want", [(36, 1), (37, 2)])
+def test_scores_given_with_many_blocks_of_d_a_warp(u, want):
+    """One kernel up to 36 expected blocks of D a warp, the pair above, and the same result."""
+    d, E, d_e, L = 256, 48, 512, 3
+    layer, dw = B.Layer(d, E, d_e, L_max=L, flags=B.cfg_expected_union(u)), make(d, E, d_e, 5, 0.0)
+    g = torch.Generator(device="cuda").manual_seed(u)
+    s, x = scores_like(L, E, g, 0.6), torch.randn(L, d, device="cuda", generator=g).bfloat16()
+    z = torch.einsum("ejd,td->tej", dw.tensors["U"].double(), x.double())
+    ref = torch.einsum("tej,ecj->tc", s.double()[:, :, None] * z * torch.sigmoid(z), dw.tensors["D"].double())
+    out = torch.empty(L, d, device="cuda")
+    torch.cuda.synchronize()
+    n0 = layer.launch_count()
+    B.blockffn_layer_forward_scores(layer.h, dw.struct, x, s, L, out, call_flags=B.CALL_INDEPENDENT)
+    assert layer.launch_count() - n0 == want and layer.last_status() == 0
+    assert (out.double() - ref).abs().max() <= 2e-2 * ref.square().mean().sqrt()
